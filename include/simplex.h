@@ -239,6 +239,11 @@ int64_t simplex_edm_tiles_len(int64_t n);
  * the denominator (cosines from the law of cosines on unsoftened squares).
  * d must be 3.  x: device, n*3 FP32.  energy: device, 1 double (written).
  * Per-triple arithmetic is FP32; the reduction across blocks is FP64.
+ * From 1664 points (up to the table limit) the sum runs as contractions of
+ * pair matrices on the tensor cores, FP16 hi + lo splits of FP32 terms with
+ * FP32 sums, over 256 x 256 super-blocks of pairs that the map's 2-simplex
+ * grid lists, and the triples of each point's nearest neighbour one by one in
+ * FP32; same accuracy or better, same workspace.
  */
 int simplex_atm_energy(int64_t n, int64_t d, const float *x, float nu, float eps,
                        double *energy, int map, void *workspace, int64_t ws_bytes,
@@ -255,7 +260,9 @@ int simplex_atm_energy(int64_t n, int64_t d, const float *x, float nu, float eps
  * aligned: the pair terms of every block pair (72 KB each, computed once per
  * call, up to 16 GB; beyond that the tiles build their own), the 16-byte
  * tile counter (zeroed by the call) and FP64 partials, one per grid block at
- * most.  Calls that share a workspace must not overlap.
+ * most.  From 640 points (while the tables fit, n <= 21,824) the sums run as
+ * contractions on the tensor cores, as in simplex_atm_energy, in the same
+ * workspace.  Calls that share a workspace must not overlap.
  */
 int simplex_atm_forces(int64_t n, int64_t d, const float *x, float nu, float eps,
                        double *energy, double *forces, int map, void *workspace,

@@ -158,7 +158,8 @@ extern "C" int simplex_device_errors(void *stream) {
     const int a = umma_device_errors(s);
     const int b = stress_umma_errors(s);
     const int c = atm_device_errors(s);
-    return a != SIMPLEX_OK ? a : (b != SIMPLEX_OK ? b : c);
+    const int d = atm_umma_errors(s);
+    return a != SIMPLEX_OK ? a : (b != SIMPLEX_OK ? b : (c != SIMPLEX_OK ? c : d));
 }
 
 extern "C" int simplex_block_rho(int op, int64_t d, int prec) {

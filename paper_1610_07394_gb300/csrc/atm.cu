@@ -1085,6 +1085,8 @@ extern "C" int simplex_atm_energy(int64_t n, int64_t d, const float *x, float nu
     double *partials = (double *)((char *)workspace + tab_bytes);
     const int64_t blocks = g.gx * g.gy * g.gz;
     double *tmp = partials + blocks;
+    if (atm_umma_energy_ok(n, tab_bytes, 8 * (blocks + kReduceSlots)))
+        return atm_umma_run(false, n, x, nu, eps, energy, nullptr, map, tab, tab_bytes, partials, s);
     if ((st = smem_optin())) return st;
     if (tab_bytes) {
         const Grid g2 = grid2(nb, map);
@@ -1126,6 +1128,9 @@ extern "C" int simplex_atm_forces(int64_t n, int64_t d, const float *x, float nu
     unsigned long long *ctr = (unsigned long long *)((char *)workspace + ftab);
     double *partials = energy ? (double *)((char *)workspace + ftab + kCounterBytes) : nullptr;
     const int64_t blocks = g.gx * g.gy * g.gz;
+    if (atm_umma_forces_ok(n, ftab, 8 * (blocks + kReduceSlots)))
+        return atm_umma_run(true, n, x, nu, eps, energy, forces, map, workspace, ftab,
+                            (char *)workspace + ftab + kCounterBytes, s);
     if ((st = cuda_status(cudaMemsetAsync(forces, 0, sizeof(double) * 3 * (size_t)n, s)))) return st;
     if ((st = cuda_status(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), s)))) return st;
     const int smem = (int)sizeof(AtmForceSmem);

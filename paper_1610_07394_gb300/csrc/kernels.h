@@ -37,4 +37,13 @@ int stress_umma_run(bool bwd, int64_t n, int64_t d, const float *x, const float 
                     cudaStream_t s);
 int stress_umma_errors(cudaStream_t s);
 
+// ATM energy and forces as contractions on the tensor cores (atm_umma.cu),
+// for the sizes whose operand tiles fit the tables' part of the workspace
+// and whose lists fit the rest.
+bool atm_umma_forces_ok(int64_t n, int64_t tab_bytes, int64_t rest_bytes);
+bool atm_umma_energy_ok(int64_t n, int64_t tab_bytes, int64_t rest_bytes);
+int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float eps, double *energy, double *forces,
+                 int map, void *tables, int64_t tab_bytes, void *rest, cudaStream_t s);
+int atm_umma_errors(cudaStream_t s);
+
 }  // namespace sx

@@ -27,6 +27,11 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n, bool a_mn_major,
            ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
+// The same with A = B = FP16 (format 0 in bits 7-9 and 10-12), both K-major.
+__host__ __device__ constexpr uint32_t idesc_f16(int m, int n) {
+    return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -200,6 +205,83 @@ __device__ __forceinline__ void mma_bf16x3_w(uint32_t tmem_d, uint64_t ah, uint6
         : "memory");
 }
 
+// kind::f16 products of a CTA pair (cta_group::2), issued by the pair's first
+// CTA from a converged warp (see mma_bf16x3_w): M = 256, 128 rows of A and of
+// D in each CTA, and the N rows of B half in each CTA, at the same shared
+// offsets.  One product D (+)= A B:
+__device__ __forceinline__ void mma2_f16_w(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred e, t;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.eq.b32 t, %3, %3;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, t;\n\t}" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc)
+        : "memory");
+}
+
+// The same with the accumulator scaled first, D = A B + 2^-SH D.
+template <int SH>
+__device__ __forceinline__ void mma2_f16_scaled_w(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred e, t;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.eq.b32 t, %3, %3;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, t, %4;\n\t}" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc), "n"(SH)
+        : "memory");
+}
+
+// The cross products of a hi + lo step, D (+)= Ah Bl + Al Bh.
+__device__ __forceinline__ void mma2_f16_cross_w(uint32_t tmem_d, uint64_t ah, uint64_t al, uint64_t bh,
+                                                 uint64_t bl, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, e, t;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.eq.b32 t, %6, %6;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %4, %5, p;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %2, %3, %5, t;\n\t}" ::"r"(tmem_d),
+        "l"(ah), "l"(al), "l"(bh), "l"(bl), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Arrives on `bar` of both CTAs of the pair once every product issued so far
+// by the elected lane has completed.
+__device__ __forceinline__ void mma2_commit_w(uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t.reg .b16 m;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "mov.b16 m, 3;\n\t"
+        "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+        " [%0], m;\n\t}" ::"r"(bar)
+        : "memory");
+}
+
+// TMEM of a CTA pair: one warp of each CTA calls these.
+__device__ __forceinline__ void tmem2_alloc(uint32_t dst_smem, uint32_t cols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem),
+                 "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem2_dealloc(uint32_t taddr, uint32_t cols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols)
+                 : "memory");
+}
+
+// Arrives on the mbarrier at `bar` of the cluster's first CTA.  What it hands
+// over is ordered by the tcgen05 fences (accumulators) or was complete before
+// (landed copies); a release at cluster scope would stall the warp for each
+// of its earlier memory accesses (a third of all stalls in the ATM kernel).
+__device__ __forceinline__ void mbar_arrive_first(uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .b32 ra;\n\t"
+        "mapa.shared::cluster.u32 ra, %0, 0;\n\t"
+        "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}" ::"r"(bar)
+        : "memory");
+}
+
 // Shared-memory matrix descriptor of an operand tile in the 128-byte swizzle
 // layout (8 rows of 128 bytes per 1024-byte atom, 16-byte chunks of row r
 // XOR-permuted by r mod 8; tile base 1024-byte aligned, so base offset 0):
@@ -305,6 +387,39 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v0)[32], float
     }
 }
 
+// 32 consecutive FP32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int t = 0; t < 32; ++t) v[t] = __uint_as_float(r[t]);
+}
+
+// Writes 32 consecutive FP32 columns of this thread's TMEM lane; complete
+// after tmem_wait_st.
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float *v) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};" ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]),
+          "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]),
+          "f"(v[16]), "f"(v[17]), "f"(v[18]), "f"(v[19]), "f"(v[20]), "f"(v[21]), "f"(v[22]), "f"(v[23]),
+          "f"(v[24]), "f"(v[25]), "f"(v[26]), "f"(v[27]), "f"(v[28]), "f"(v[29]), "f"(v[30]), "f"(v[31]),
+        "r"(taddr)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 // 16 consecutive FP32 columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
@@ -398,7 +513,21 @@ inline bool make_map_bf16(CUtensorMap *m, void *ptr, int64_t rows, int64_t cols,
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The same map with boxes of 32 BF16 (64 bytes) per row in the 64-byte swizzle.
+// `rows` rows of 64 16-bit elements (128 bytes, base 16-byte aligned), boxes
+// of box_rows whole rows, copied as they lie (no swizzle).
+inline bool make_map_rows16(CUtensorMap *m, void *ptr, int64_t rows, int box_rows) {
+    EncodeTiled f = encode_fn();
+    if (!f) return false;
+    const cuuint64_t dims[2] = {64u, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {128u};
+    const cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    return f(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ptr, dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The map of make_map_bf16 with boxes of 32 BF16 (64 bytes) per row in the 64-byte swizzle.
 inline bool make_map_bf16_sw64(CUtensorMap *m, void *ptr, int64_t rows, int64_t cols, int64_t pitch,
                                int box_rows) {
     EncodeTiled f = encode_fn();
