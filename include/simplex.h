@@ -72,7 +72,9 @@ typedef enum {
 } simplex_map;
 
 typedef enum {
-    SIMPLEX_PREC_FP32 = 0,    /* every step in FP32 (difference form)        */
+    SIMPLEX_PREC_FP32 = 0,    /* FP32 accuracy: every step in FP32, or for the
+                                 stress at size FP16 hi + lo products that err
+                                 no more (simplex_stress_fwd)                */
     SIMPLEX_PREC_BF16X3 = 1,  /* Gram term on tensor cores, split BF16 hi+lo */
     SIMPLEX_PREC_AUTO = 2     /* library choice by d                          */
 } simplex_prec;
@@ -273,6 +275,11 @@ int simplex_atm_forces(int64_t n, int64_t d, const float *x, float nu, float eps
  * D_ij = |x_i - x_j|^2 and delta_ij = |y_i - y_j|^2 recomputed from y.
  * x, y: device, n*d FP32.  d_out: device, n(n+1)/2 FP32, or NULL to skip
  * storing D.  loss: device, 1 double (written).
+ * prec FP32: from about n^2 (d + 20) = 2e8 (gradient) or 3.6e8 (loss), d <= 96
+ * and no d_out, the pair products run on the tensor cores from FP16 hi + lo
+ * splits on a fixed grid (22 bits and more) with FP32 sums, where the workspace
+ * has simplex_workspace_bytes(); with less (8 bytes per grid block and 1024 for
+ * a loss, none for the gradient alone) every step stays in FP32.
  */
 int simplex_stress_fwd(int64_t n, int64_t d, const float *x, const float *y,
                        float *d_out, double *loss, int map, int prec,

@@ -191,15 +191,20 @@ extern "C" int64_t simplex_workspace_bytes(int op, int64_t n, int64_t d, int map
             if (stress_use_umma(d, prec)) return stress_umma_workspace_bytes(n, d, false);
             const int64_t nb = (n + kStressRho - 1) / kStressRho;
             const Grid g = grid2(nb, map);
-            return 8 * (g.gx * g.gy * g.gz + kReduceSlots);
+            const int64_t simt = 8 * (g.gx * g.gy * g.gz + kReduceSlots);
+            const int64_t f16 = stress_f16_ok(n, d, false) ? stress_f16_workspace_bytes(n, d, false) : 0;
+            return simt > f16 ? simt : f16;
         }
         case SIMPLEX_OP_STRESS_BWD:
-            return stress_use_umma(d, prec) ? stress_umma_workspace_bytes(n, d, true) : 0;
+            if (stress_use_umma(d, prec)) return stress_umma_workspace_bytes(n, d, true);
+            return stress_f16_ok(n, d, true) ? stress_f16_workspace_bytes(n, d, true) : 0;
         case SIMPLEX_OP_STRESS_FWD_BWD: {
             if (stress_use_umma(d, prec)) return stress_umma_workspace_bytes(n, d, true);
             const int64_t nb = (n + kStressRho - 1) / kStressRho;
             const Grid g = grid2(nb, map);
-            return 8 * (g.gx * g.gy + kReduceSlots);
+            const int64_t simt = 8 * (g.gx * g.gy + kReduceSlots);
+            const int64_t f16 = stress_f16_ok(n, d, true) ? stress_f16_workspace_bytes(n, d, true) : 0;
+            return simt > f16 ? simt : f16;
         }
         default: return -1;
     }

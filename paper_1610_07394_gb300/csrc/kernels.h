@@ -37,6 +37,14 @@ int stress_umma_run(bool bwd, int64_t n, int64_t d, const float *x, const float 
                     cudaStream_t s);
 int stress_umma_errors(cudaStream_t s);
 
+// SIMPLEX_PREC_FP32 on the same kernels with FP16 hi + lo operands (d <= 96):
+// by size, with a workspace of this many bytes (the FP32 kernels of stress.cu
+// otherwise).
+bool stress_f16_ok(int64_t n, int64_t d, bool bwd);
+int64_t stress_f16_workspace_bytes(int64_t n, int64_t d, bool bwd);
+int stress_f16_run(bool bwd, int64_t n, int64_t d, const float *x, const float *y, double *loss, double gscale,
+                   float *grad, int map, void *ws, cudaStream_t s);
+
 // ATM energy and forces as contractions on the tensor cores (atm_umma.cu),
 // for the sizes whose operand tiles fit the tables' part of the workspace
 // and whose lists fit the rest.

@@ -296,6 +296,13 @@ static int stress_check(int64_t n, int64_t d, const float *x, const float *y, in
     return SIMPLEX_OK;
 }
 
+// FP32 on the tensor cores: by size, where the caller's workspace has room
+// for the operands (a smaller one, or none where none was asked for before,
+// keeps the FP32 kernels).
+static bool use_f16(int64_t n, int64_t d, bool bwd, const void *ws, int64_t ws_bytes) {
+    return stress_f16_ok(n, d, bwd) && ws && aligned(ws, 256) && ws_bytes >= stress_f16_workspace_bytes(n, d, bwd);
+}
+
 constexpr int kStressSmem = (int)sizeof(StressSmem);
 
 // The tile's shared memory exceeds the 48 KB default of a launch; opt in
@@ -341,6 +348,8 @@ extern "C" int simplex_stress_fwd(int64_t n, int64_t d, const float *x, const fl
     const int64_t blocks = g.gx * g.gy;
     if (!workspace || ws_bytes < 8 * (blocks + kReduceSlots) || !aligned(workspace, 256))
         return SIMPLEX_EWORKSPACE;
+    if (!d_out && use_f16(n, d, false, workspace, ws_bytes))
+        return stress_f16_run(false, n, d, x, y, loss, 0.0, nullptr, map, workspace, (cudaStream_t)stream);
     if ((st = stress_optin())) return st;
     cudaStream_t s = (cudaStream_t)stream;
     double *partials = (double *)workspace;
@@ -375,6 +384,8 @@ static int stress_grad(int64_t n, int64_t d, const float *x, const float *y, dou
             return SIMPLEX_EWORKSPACE;
         partials = (double *)workspace;
     }
+    if (use_f16(n, d, true, workspace, ws_bytes))
+        return stress_f16_run(true, n, d, x, y, loss, gscale, grad, map, workspace, s);
     if ((st = stress_optin())) return st;
     if ((st = cuda_status(cudaMemsetAsync(grad, 0, sizeof(float) * (size_t)(n * d), s)))) return st;
     const float scale4 = (float)(4.0 * gscale);

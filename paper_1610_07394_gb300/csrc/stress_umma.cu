@@ -39,6 +39,8 @@
 // issues the MMAs (the accumulation of step t+1 runs while the epilogue
 // drains step t), eight epilogue warps (two per TMEM lane quarter) read the
 // accumulators.  Every wait is bounded (simplex_device_errors).
+#include <cuda_fp16.h>
+
 #include <cstddef>
 #include <mutex>
 
@@ -245,6 +247,107 @@ struct ChunkWalk {
     }
 };
 
+// ---------------------------------------------------------------- FP32 on the tensor cores
+//
+// SIMPLEX_PREC_FP32 with the products on the tensor cores (F16 = true): the
+// operands are split into FP16 hi + lo on one fixed grid each.  S is scaled by
+// the power of two that takes the largest |S| of all points to [2^10, 2^11),
+// hi = the nearest integer (11 bits, exact in FP16), lo = the rest rounded to
+// 11 bits: 2^-24 of that largest; Delta likewise.  hi.hi is then a sum of
+// integers, exact in the tensor core's truncating FP32 sums up to 2^24, and
+// has an accumulator of its own; the three other products, 2^-11 of it, have
+// another.  So the residuals carry no truncation (in one accumulator all of M
+// came out 1e-7 small, and the loss with it).  The second product's operands
+// (the residual tile C, X) are rounded to FP16 hi + lo of 22 bits, scaled into
+// FP16's range by bounds on |r| and |x|; both sides are flushed for every
+// tile, so that no truncating sum runs over more than 128 points.  The
+// residuals and the gradient do not change when x and y move together, so
+// both are taken from a centre c (the mean of 64 points): the products' size
+// is then the cloud's, wherever it lies.  Against 64 bits, N(0,1) clouds of
+// n = 2560 to 20000, d = 2 to 96: loss 1e-10 to 5e-9 as with the FP32 kernels,
+// gradient 1.0e-7 to 2.0e-7 of its norm (1.0e-7 to 2.9e-7); a cloud 20 times its
+// width away from the origin 1e-7 to 2e-7 (6e-7 to 1.7e-6).
+constexpr int kCentre = 64;   // points of the mean
+constexpr int kMaxDim = 96;
+
+struct Scales {
+    float s, d, x, c;        // of S, Delta, x and the residuals
+    float is, id, ix, ic;    // their inverses
+};
+
+// mx: the bits of the largest |S|, |Delta|, |x|.
+__device__ __forceinline__ float pow2_scale(float m, int top) {
+    int e = 0;
+    if (m > 0.f && m <= 3.4e38f) frexpf(m, &e);   // m < 2^e; 0, inf and NaN take 1
+    e = top - e;
+    return ldexpf(1.0f, e > 100 ? 100 : (e < -100 ? -100 : e));
+}
+
+__device__ __forceinline__ Scales scales_of(const uint32_t *mx, int d) {
+    const float ms = __uint_as_float(__ldg(mx)), md = __uint_as_float(__ldg(mx + 1)), mxx = __uint_as_float(__ldg(mx + 2));
+    Scales q;
+    q.s = pow2_scale(ms, 11);
+    q.d = pow2_scale(md, 11);
+    q.x = pow2_scale(mxx, 11);
+    // |r| <= 4 d max|S| max|Delta| < 2^15 / c
+    int es = 0, ed = 0;
+    if (ms > 0.f && ms <= 3.4e38f) frexpf(ms, &es);
+    if (md > 0.f && md <= 3.4e38f) frexpf(md, &ed);
+    int e = 15 - (es + ed + 2 + (32 - __clz(d)));
+    q.c = ldexpf(1.0f, e > 100 ? 100 : (e < -100 ? -100 : e));
+    q.is = 1.0f / q.s; q.id = 1.0f / q.d; q.ix = 1.0f / q.x; q.ic = 1.0f / q.c;
+    return q;
+}
+
+// c, and zeroed maxima (one block of 8 x 96 threads).
+__global__ void __launch_bounds__(8 * kMaxDim) k_stress_centre(const float *__restrict__ x, int64_t n, int d,
+                                                               float *__restrict__ c, uint32_t *__restrict__ mx) {
+    __shared__ float part[8][kMaxDim];
+    const int t = threadIdx.x % kMaxDim, g = threadIdx.x / kMaxDim;
+    float v = 0.f;
+    if (t < d)
+        for (int k = g; k < kCentre; k += 8) v += __ldg(x + (n * k / kCentre) * d + t) * (1.0f / kCentre);
+    part[g][t] = v;
+    __syncthreads();
+    if (g == 0) {
+#pragma unroll
+        for (int k = 1; k < 8; ++k) v += part[k][t];
+        c[t] = v;
+    }
+    if (threadIdx.x < 3) mx[threadIdx.x] = 0u;
+}
+
+// Largest |S|, |Delta|, |x - c| (as bits: NaN above infinity above all numbers).
+__global__ void __launch_bounds__(256) k_stress_max(const float *__restrict__ x, const float *__restrict__ y,
+                                                    int64_t count, int d, const float *__restrict__ c,
+                                                    uint32_t *__restrict__ mx) {
+    uint32_t m[3] = {0u, 0u, 0u};
+    const int64_t e0 = (int64_t)blockIdx.x * 256 + threadIdx.x, step = (int64_t)gridDim.x * 256;
+    int t = (int)(e0 % d);
+    const int dt = (int)(step % d);
+    for (int64_t e = e0; e < count; e += step) {
+        const float ct = __ldg(c + t), a = __ldg(x + e), b = __ldg(y + e);
+        m[0] = max(m[0], __float_as_uint(fabsf((a - ct) + (b - ct))));
+        m[1] = max(m[1], __float_as_uint(fabsf(a - b)));
+        m[2] = max(m[2], __float_as_uint(fabsf(a - ct)));
+        t += dt;
+        if (t >= d) t -= d;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        m[k] = __reduce_max_sync(0xffffffffu, m[k]);
+        if ((threadIdx.x & 31) == 0 && m[k]) atomicMax(mx + k, m[k]);
+    }
+}
+
+// hi and lo of a value on the integer grid.
+__device__ __forceinline__ void split_grid(float v, uint16_t &h, uint16_t &l) {
+    const float r = rintf(v);
+    const __half hh = __float2half_rn(r), ll = __float2half_rn(v - r);
+    h = __half_as_ushort(hh);
+    l = __half_as_ushort(ll);
+}
+
 // Next ring stage for the producer: waits until it is free and arms it for
 // `bytes` of TMA data.
 template <int S>
@@ -288,25 +391,55 @@ __device__ __forceinline__ void load_xt(const CUtensorMap *mh, const CUtensorMap
 // scale4 S_p x_p (k_stress_sx), so no coordinate is loaded here.  This
 // thread: its lane quarter's row, its half of the d coordinates (the sum
 // once, by half 0).  All lanes execute the TMEM loads.
+// F16: dp columns in the accumulator (d of them coordinates, any row
+// alignment), in units of 1/gs (coordinates) and 1/ss (sums).
+template <bool F16>
 __device__ __forceinline__ void flush_g(uint32_t tmem, uint32_t gcol, int B, int quarter, int half,
-                                        int lane, int d, int64_t n, float scale4, float *__restrict__ grad,
-                                        float *__restrict__ S) {
+                                        int lane, int d, int dp, int64_t n, float scale4, float gs, float ss,
+                                        float *__restrict__ grad, float *__restrict__ S) {
     const uint32_t tl = tmem + ((uint32_t)(32 * quarter) << 16) + gcol;
-    const float s = tmem_ld1(tl + (uint32_t)d);
+    const float s = tmem_ld1(tl + (uint32_t)dp);
     const int64_t row = (int64_t)B * TM + 32 * quarter + lane;
-    const int hw = d >> 1;
+    const int hw = dp >> 1;
+    // F16: the truncating sums come out 2e-8 (d >= 16) to 6e-8 (d = 2) small,
+    // measured against 64 bits; this share of each gives the mean back
+    constexpr float kShare = 3.5e-8f;
+    const float f = F16 ? -scale4 * gs : -scale4, fs = f * kShare;
     for (int c = 0; c < hw; c += 16) {
         float v[16];
         tmem_ld16(tl + (uint32_t)(half * hw + c), v);
+        const int c0 = half * hw + c;
         if (row < n) {
-            float *gr = grad + row * d + half * hw + c;
+            if (F16)
 #pragma unroll
-            for (int q = 0; q < 16; q += 4)
-                atomicAdd(reinterpret_cast<float4 *>(gr + q),
-                          make_float4(-scale4 * v[q], -scale4 * v[q + 1], -scale4 * v[q + 2], -scale4 * v[q + 3]));
+                for (int q = 0; q < 16; ++q) v[q] = fmaf(v[q], f, v[q] * fs);
+            else
+#pragma unroll
+                for (int q = 0; q < 16; ++q) v[q] *= f;
+            float *gr = grad + row * d + c0;
+            if (!F16 || ((d & 3) == 0 && c0 + 16 <= d)) {
+#pragma unroll
+                for (int q = 0; q < 16; q += 4)
+                    atomicAdd(reinterpret_cast<float4 *>(gr + q),
+                              make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]));
+            } else {
+#pragma unroll
+                for (int q = 0; q < 16; ++q)
+                    if (c0 + q < d) atomicAdd(gr + q, v[q]);
+            }
         }
     }
-    if (half == 0 && row < n) atomicAdd(S + row, s);
+    if (half == 0 && row < n) atomicAdd(S + row, F16 ? fmaf(s, ss, s * (ss * kShare)) : s);
+}
+
+// The same from the centre, one element at a time (any d, any alignment of x).
+__global__ void __launch_bounds__(256) k_stress_sx_centred(const float *__restrict__ x, const float *__restrict__ c,
+                                                           const float *__restrict__ S, int64_t n, int d, float scale4,
+                                                           float *__restrict__ grad) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n * d) return;
+    const int64_t p = e / d;
+    grad[e] = fmaf(scale4 * S[p], __ldg(x + e) - __ldg(c + (e - p * d)), grad[e]);
 }
 
 // grad_p += scale4 S_p x_p, the row-sum part of every flush (see flush_g).
@@ -340,14 +473,18 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 // The backward kernel (gradient): 128 x 128 tiles, GEMM1 then GEMM2.  With
 // `partials` it also sums the loss from the same residual tiles (one FP64
 // partial per CTA): loss and gradient in one pass.
-template <int MAP>
+template <int MAP, bool F16>
 __global__ void __launch_bounds__(kThreads, 1)
     k_stress_umma_bwd(const __grid_constant__ CUtensorMap mPh, const __grid_constant__ CUtensorMap mPl,
                       const __grid_constant__ CUtensorMap mQh, const __grid_constant__ CUtensorMap mQl,
                       const __grid_constant__ CUtensorMap mTh, const __grid_constant__ CUtensorMap mTl,
                       float *__restrict__ S, const float *__restrict__ a, int64_t n, int d, int nb,
                       int gx, int64_t T, int64_t nchunks, const int64_t *__restrict__ start,
-                      float scale4, float *__restrict__ grad, double *__restrict__ partials, int qshift) {
+                      float scale4, float *__restrict__ grad, double *__restrict__ partials, int qshift, int dg,
+                      const uint32_t *__restrict__ mx) {
+    // d: coordinates in the operands (a multiple of 32), dg: in grad.
+    // GEMM1 accumulators: two, used in turn (BF16), or one pair hi.hi | rest (F16)
+    constexpr uint32_t kAcc = F16 ? 1 : 2;
     using Walk = ChunkWalk<MAP>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
@@ -437,9 +574,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // warps and a 128 x 80 x 16 MMA of GEMM2 runs about 40 cycles, so the
         // instructions between MMAs decide whether the tensor pipe idles.
         {
-            const uint32_t id1 = idesc_bf16(TM, TN, false, false);
-            const uint32_t id_row = idesc_bf16(TM, NG, false, false);
-            const uint32_t id_col = idesc_bf16(TM, NG, true, false);
+            const uint32_t id1 = F16 ? idesc_f16(TM, TN) : idesc_bf16(TM, TN, false, false);
+            const uint32_t id_row = F16 ? idesc_f16(TM, NG) : idesc_bf16(TM, NG, false, false);
+            const uint32_t id_col = F16 ? idesc_f16(TM, NG, true) : idesc_bf16(TM, NG, true, false);
             const uint64_t dc = sw128_desc(s_c);                     // C, K-major (rows side)
             const uint64_t dct = sw128_desc(s_c, TILE_BYTES, 1024);  // C read M-major (columns side)
             Walk walk(gx, nb, T, nchunks, start);
@@ -466,28 +603,58 @@ __global__ void __launch_bounds__(kThreads, 1)
                 // rows: G_Y (+)= C [X_X | 1], K = j over the two column halves of C
                 if (!ring_take<NS>(ctl, s_stages, it, src, fail)) return false;
                 const uint64_t dx = sw128_desc(src);
+                if (F16) {   // the cross products first, while the sums are small
 #pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int ks = 0; ks < KC / 16; ++ks) {
-                        const uint32_t acc = (h == 0 && ks == 0 && !sameY) ? 0u : 1u;
-                        mma_bf16x3_w(tmem + kGY, desc_add(dc, h * TILE_BYTES + ks * 32),
-                                     desc_add(dc, (2 + h) * TILE_BYTES + ks * 32),
-                                     desc_add(dx, h * xt_box + ks * 32), desc_add(dx, (2 + h) * xt_box + ks * 32),
-                                     id_row, acc);
+                    for (int ks = 0; ks < TN / 16; ++ks) {
+                        const uint32_t h = (uint32_t)(ks >> 2), ko = (uint32_t)(ks & 3) * 32;
+                        mma_cross_w(tmem + kGY, desc_add(dc, h * TILE_BYTES + ko), desc_add(dc, (2 + h) * TILE_BYTES + ko),
+                                    desc_add(dx, h * xt_box + ko), desc_add(dx, (2 + h) * xt_box + ko), id_row,
+                                    ks ? 1u : 0u);
                     }
+#pragma unroll
+                    for (int ks = 0; ks < TN / 16; ++ks) {
+                        const uint32_t h = (uint32_t)(ks >> 2), ko = (uint32_t)(ks & 3) * 32;
+                        mma_add_w(tmem + kGY, desc_add(dc, h * TILE_BYTES + ko), desc_add(dx, h * xt_box + ko), id_row);
+                    }
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int ks = 0; ks < KC / 16; ++ks) {
+                            const uint32_t acc = (h == 0 && ks == 0 && !sameY) ? 0u : 1u;
+                            mma_bf16x3_w(tmem + kGY, desc_add(dc, h * TILE_BYTES + ks * 32),
+                                         desc_add(dc, (2 + h) * TILE_BYTES + ks * 32),
+                                         desc_add(dx, h * xt_box + ks * 32), desc_add(dx, (2 + h) * xt_box + ks * 32),
+                                         id_row, acc);
+                        }
+                }
                 mma_commit_w(smem_u32(&ctl.empty[it % NS]));
                 ++it;
                 // columns: G_X = C^T [X_Y | 1], K = i; A is C read M-major (M = j
                 // over the two 64-column halves, LBO = one half tile apart)
                 if (!ring_take<NS>(ctl, s_stages, it, src, fail)) return false;
                 const uint64_t dy = sw128_desc(src);
+                if (F16) {
 #pragma unroll
-                for (int ks = 0; ks < TM / 16; ++ks) {
-                    const uint32_t hb = (uint32_t)(ks >> 2), kb = (uint32_t)(ks & 3) * 32;
-                    mma_bf16x3_w(tgx, desc_add(dct, ks * 2048), desc_add(dct, 2 * TILE_BYTES + ks * 2048),
-                                 desc_add(dy, hb * xt_box + kb), desc_add(dy, (2 + hb) * xt_box + kb), id_col,
-                                 ks ? 1u : 0u);
+                    for (int ks = 0; ks < TM / 16; ++ks) {
+                        const uint32_t hb = (uint32_t)(ks >> 2), kb = (uint32_t)(ks & 3) * 32;
+                        mma_cross_w(tgx, desc_add(dct, ks * 2048), desc_add(dct, 2 * TILE_BYTES + ks * 2048),
+                                    desc_add(dy, hb * xt_box + kb), desc_add(dy, (2 + hb) * xt_box + kb), id_col,
+                                    ks ? 1u : 0u);
+                    }
+#pragma unroll
+                    for (int ks = 0; ks < TM / 16; ++ks) {
+                        const uint32_t hb = (uint32_t)(ks >> 2), kb = (uint32_t)(ks & 3) * 32;
+                        mma_add_w(tgx, desc_add(dct, ks * 2048), desc_add(dy, hb * xt_box + kb), id_col);
+                    }
+                } else {
+#pragma unroll
+                    for (int ks = 0; ks < TM / 16; ++ks) {
+                        const uint32_t hb = (uint32_t)(ks >> 2), kb = (uint32_t)(ks & 3) * 32;
+                        mma_bf16x3_w(tgx, desc_add(dct, ks * 2048), desc_add(dct, 2 * TILE_BYTES + ks * 2048),
+                                     desc_add(dy, hb * xt_box + kb), desc_add(dy, (2 + hb) * xt_box + kb), id_col,
+                                     ks ? 1u : 0u);
+                    }
                 }
                 mma_commit_w(smem_u32(&ctl.empty[it % NS]));
                 ++it;
@@ -495,7 +662,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 return true;
             };
             while (ok && !*fail && walk.next(X, Y)) {
-                const uint32_t acc = t & 1, aph = (t >> 1) & 1;
+                const uint32_t acc = t % kAcc, aph = (t / kAcc) & 1;
                 if (!(ok = mbar_wait(smem_u32(&ctl.tempty[acc]), aph ^ 1, fail, &g_error))) break;
                 tc_fence_after();
                 const uint32_t dtm = tmem + acc * TN;
@@ -504,22 +671,25 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const uint64_t d0 = sw128_desc(src);   // P hi, P lo, Q hi, Q lo tiles of the stage
 #pragma unroll
                     for (int ks = 0; ks < KC / 16; ++ks) {
-                        const uint32_t ko = ks * 32;
-                        mma_bf16x3_w(dtm, desc_add(d0, ko), desc_add(d0, TILE_BYTES + ko),
-                                     desc_add(d0, 2 * TILE_BYTES + ko), desc_add(d0, 3 * TILE_BYTES + ko), id1,
-                                     (c > 0 || ks > 0) ? 1u : 0u);
+                        const uint32_t ko = ks * 32, more = (c > 0 || ks > 0) ? 1u : 0u;
+                        if (F16)
+                            mma_split4_w(dtm, dtm + TN, desc_add(d0, ko), desc_add(d0, TILE_BYTES + ko),
+                                         desc_add(d0, 2 * TILE_BYTES + ko), desc_add(d0, 3 * TILE_BYTES + ko), id1, more);
+                        else
+                            mma_bf16x3_w(dtm, desc_add(d0, ko), desc_add(d0, TILE_BYTES + ko),
+                                         desc_add(d0, 2 * TILE_BYTES + ko), desc_add(d0, 3 * TILE_BYTES + ko), id1, more);
                     }
                     mma_commit_w(smem_u32(&ctl.empty[it % NS]));
                     ++it;
                 }
                 if (!ok) break;
                 mma_commit_w(smem_u32(&ctl.tfull[acc]));
-                if (t >= 1 && !(ok = gemm2(t - 1, t >= 2 && prevY == prev2Y))) break;
+                if (t >= 1 && !(ok = gemm2(t - 1, !F16 && t >= 2 && prevY == prev2Y))) break;
                 prev2Y = prevY;
                 prevY = Y;
                 ++t;
             }
-            if (ok && !*fail && t >= 1) gemm2(t - 1, t >= 2 && prevY == prev2Y);
+            if (ok && !*fail && t >= 1) gemm2(t - 1, !F16 && t >= 2 && prevY == prev2Y);
             // everything issued has completed before the block releases TMEM
             mma_commit_w(smem_u32(&ctl.done));
             mbar_drain(smem_u32(&ctl.done), 0);
@@ -534,6 +704,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int ngx = gx_buffers(NG);
         unsigned char *rowh = cbuf + half * TILE_BYTES + (r >> 3) * 1024 + (r & 7) * 128;
         unsigned char *rowl = rowh + 2 * TILE_BYTES;
+        Scales sc = {};
+        if (F16) sc = scales_of(mx, dg);
+        const float gs = sc.ix * sc.ic, ss = sc.ic;
         Walk walk(gx, nb, T, nchunks, start);
         uint32_t t = 0;
         int X, Y, pX = 0, pY = 0;
@@ -546,7 +719,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const bool hn = walk.next(Xn, Yn);
             float na = 0.f, nbv = 0.f, ni = 0.f;
             if (hn) load_a(a, n, Xn, Yn, half, r, lane, na, nbv, ni);
-            const uint32_t acc = t & 1, aph = (t >> 1) & 1;
+            const uint32_t acc = t % kAcc, aph = (t / kAcc) & 1;
             const int64_t row0 = (int64_t)Y * TM, jb = (int64_t)X * TN + 64 * half;
             __syncwarp();   // the previous tile's reads of ac are done
             ac[lane] = va;
@@ -564,9 +737,19 @@ __global__ void __launch_bounds__(kThreads, 1)
             {
                 float v0[32], v1[32];
                 const uint32_t taddr = tmem + acc * TN + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(64 * half);
-                tmem_ld64(taddr, v0, v1);
+                if (F16) {   // hi.hi, then the other products' accumulator
 #pragma unroll
-                for (int q = 0; q < 32; ++q) { v[q] = v0[q]; v[32 + q] = v1[q]; }
+                    for (int p = 0; p < 64; p += 32) {
+                        tmem_ld32(taddr + p, v0);
+                        tmem_ld32(taddr + TN + p, v1);
+#pragma unroll
+                        for (int q = 0; q < 32; ++q) v[p + q] = ((v0[q] + v1[q]) * sc.is) * sc.id;
+                    }
+                } else {
+                    tmem_ld64(taddr, v0, v1);
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) { v[q] = v0[q]; v[32 + q] = v1[q]; }
+                }
             }
             tc_fence_before();
             __syncwarp();
@@ -595,7 +778,16 @@ __global__ void __launch_bounds__(kThreads, 1)
                 uint32_t ph[4], pl[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const float f0 = v[8 * c + 2 * k], f1 = v[8 * c + 2 * k + 1];
+                    const float f0 = F16 ? v[8 * c + 2 * k] * sc.c : v[8 * c + 2 * k],
+                                f1 = F16 ? v[8 * c + 2 * k + 1] * sc.c : v[8 * c + 2 * k + 1];
+                    if (F16) {
+                        const __half2 hf = __floats2half2_rn(f0, f1);
+                        const float2 b = __half22float2(hf);
+                        const __half2 lf = __floats2half2_rn(f0 - b.x, f1 - b.y);
+                        ph[k] = *reinterpret_cast<const uint32_t *>(&hf);
+                        pl[k] = *reinterpret_cast<const uint32_t *>(&lf);
+                        continue;
+                    }
                     const __nv_bfloat162 hh = __floats2bfloat162_rn(f0, f1);   // both rounded at once
                     ph[k] = *reinterpret_cast<const uint32_t *>(&hh);
                     pl[k] = pack_bf16(f0 - __low2float(hh), f1 - __high2float(hh));
@@ -610,12 +802,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (t >= 1) {
                 // the previous tile's sides: its columns always, its rows at the end of a run
                 const uint32_t pb = (t - 1) % (uint32_t)ngx;
-                flush_g(tmem, kGY + NG * (1 + pb), pX, quarter, half, lane, d, n, scale4, grad, S);
+                flush_g<F16>(tmem, kGY + NG * (1 + pb), pX, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctl.gxfree[pb]));
-                if (Y != pY) {
-                    flush_g(tmem, kGY, pY, quarter, half, lane, d, n, scale4, grad, S);
+                if (F16 || Y != pY) {
+                    flush_g<F16>(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&ctl.gyfree));
@@ -630,9 +822,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!*fail && t >= 1 &&
             mbar_wait(smem_u32(&ctl.g2done), (t - 1) & 1, fail, &g_error)) {
             tc_fence_after();
-            flush_g(tmem, kGY + NG * (1 + (t - 1) % (uint32_t)ngx), pX, quarter, half, lane, d, n, scale4,
-                    grad, S);
-            flush_g(tmem, kGY, pY, quarter, half, lane, d, n, scale4, grad, S);
+            flush_g<F16>(tmem, kGY + NG * (1 + (t - 1) % (uint32_t)ngx), pX, quarter, half, lane, dg, d, n, scale4, gs,
+                         ss, grad, S);
+            flush_g<F16>(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
         }
     }
     tc_fence_before();
@@ -683,12 +875,15 @@ static_assert(sizeof(Ctl2) <= kCtl2Bytes, "control block");
 static_assert(SMEM2 <= 227 * 1024, "shared memory per block");
 static_assert(2 * TN2 <= kTmemCols, "two accumulators of 256 columns");
 
-template <int MAP>
+template <int MAP, bool F16>
 __global__ void __launch_bounds__(kThreads, 1)
     k_stress_umma_fwd(const __grid_constant__ CUtensorMap mPh, const __grid_constant__ CUtensorMap mPl,
                     const __grid_constant__ CUtensorMap mQh, const __grid_constant__ CUtensorMap mQl,
                     const float *__restrict__ a, int64_t n, int d, int nb, int nb2, int gx,
-                    int64_t total, double *__restrict__ partials, int qshift) {
+                    int64_t total, double *__restrict__ partials, int qshift, int dg,
+                    const uint32_t *__restrict__ mx) {
+    // accumulators: two, used in turn (BF16), or one pair hi.hi | rest (F16)
+    constexpr uint32_t kAcc = F16 ? 1 : 2;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -757,13 +952,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (warp == 1) {
         // ---------------- MMA issuer
         {   // the whole warp, converged; one elected lane issues
-            const uint32_t id = idesc_bf16(TM, TN2, false, false);
+            const uint32_t id = F16 ? idesc_f16(TM, TN2) : idesc_bf16(TM, TN2, false, false);
             SuperWalk<MAP> walk(gx, total, nb2);
             uint32_t it = 0, t = 0;
             int sX, sY;
             bool ok = true;
             while (ok && !*fail && walk.next(sX, sY)) {
-                const uint32_t acc = t & 1, aph = (t >> 1) & 1;
+                const uint32_t acc = t % kAcc, aph = (t / kAcc) & 1;
                 if (!(ok = mbar_wait(smem_u32(&ctl.tempty[acc]), aph ^ 1, fail, &g_error))) break;
                 tc_fence_after();
                 const uint32_t dtm = tmem + acc * TN2;
@@ -775,9 +970,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const uint64_t d0 = sw128_desc(src);
 #pragma unroll
                     for (int ks = 0; ks < KC / 16; ++ks) {
-                        const uint32_t ko = ks * 32;
-                        mma_bf16x3_w(dtm, desc_add(d0, ko), desc_add(d0, A_BYTES + ko), desc_add(d0, 2 * A_BYTES + ko),
-                                     desc_add(d0, 2 * A_BYTES + B_BYTES + ko), id, (c > 0 || ks > 0) ? 1u : 0u);
+                        const uint32_t ko = ks * 32, more = (c > 0 || ks > 0) ? 1u : 0u;
+                        if (F16)
+                            mma_split4_w(dtm, dtm + TN2, desc_add(d0, ko), desc_add(d0, A_BYTES + ko),
+                                         desc_add(d0, 2 * A_BYTES + ko), desc_add(d0, 2 * A_BYTES + B_BYTES + ko), id, more);
+                        else
+                            mma_bf16x3_w(dtm, desc_add(d0, ko), desc_add(d0, A_BYTES + ko), desc_add(d0, 2 * A_BYTES + ko),
+                                         desc_add(d0, 2 * A_BYTES + B_BYTES + ko), id, more);
                     }
                     // the stage is free once this CTA's MMAs and the peer's have read it
                     mma_commit_mc_w(smem_u32(&ctl.empty[s]), 3);
@@ -799,12 +998,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int h = ew >> 2;                   // column block 2 sX + h: accumulator columns 128 h ..
         const int r = 32 * quarter + lane;       // this thread's row in the tile
         float *ac = &ctl.acol[ew][0];
+        Scales sc = {};
+        if (F16) sc = scales_of(mx, dg);
         SuperWalk<MAP> walk(gx, total, nb2);
         uint32_t t = 0;
         int sX, sY;
         while (!*fail && walk.next(sX, sY)) {
             const int Y = 2 * sY + (int)rank, X = 2 * sX + h;
-            const uint32_t acc = t & 1, aph = (t >> 1) & 1;
+            const uint32_t acc = t % kAcc, aph = (t / kAcc) & 1;
             const int64_t i = (int64_t)Y * TM + r, jb = (int64_t)X * TN;
             __syncwarp();   // the previous step's reads of ac are done
 #pragma unroll
@@ -828,6 +1029,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint32_t taddr = tmem + acc * TN2 + ((uint32_t)(32 * quarter) << 16) +
                                        (uint32_t)(TN * h + 64 * part);
                 tmem_ld64(taddr, v0, v1);
+                if (F16) {   // the other products' accumulator, 32 columns at a time
+                    float w[32];
+                    tmem_ld32(taddr + TN2, w);
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) v0[q] = ((v0[q] + w[q]) * sc.is) * sc.id;
+                    tmem_ld32(taddr + TN2 + 32, w);
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) v1[q] = ((v1[q] + w[q]) * sc.is) * sc.id;
+                }
 #pragma unroll
                 for (int q = 0; q < 32; q += 4) {
                     const int c0 = 64 * part + q;
@@ -868,37 +1078,64 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace f256
 
-// P = [S | Delta], Q = [Delta | S] (BF16 hi, lo; rows of 2d; Q only when
-// Qh is given), a = S . Delta in FP32, and for the backward pass X^T hi, lo (rows t < d: coordinates; row d:
-// ones; rows d+1 .. NG-1: zeros; row pitch `pitch`).  32 points per block.
+// hi and lo of a value, BF16 or (F16) FP16 of a scaled value.
+template <bool F16>
+__device__ __forceinline__ void split_float(float v, uint16_t &h, uint16_t &l) {
+    if (F16) {
+        const __half hh = __float2half_rn(v);
+        h = __half_as_ushort(hh);
+        l = __half_as_ushort(__float2half_rn(v - __half2float(hh)));
+    } else {
+        const __nv_bfloat16 hh = __float2bfloat16_rn(v);
+        h = __bfloat16_as_ushort(hh);
+        l = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(hh)));
+    }
+}
+
+// P = [S | Delta], Q = [Delta | S] (hi, lo; rows of 2 dp; Q only when Qh is
+// given), a = S . Delta in FP32, and for the backward pass X^T hi, lo (rows
+// t < d: coordinates; row dp: ones; the others up to NG - 1: zeros; row pitch
+// `pitch`).  dp = d for BF16; for FP16 (F16) the next multiple of 32, the
+// columns beyond d zero.  32 points per block.
+template <bool F16>
 __global__ void __launch_bounds__(256) k_stress_prep(const float *__restrict__ x,
-                                                     const float *__restrict__ y, int64_t n, int d,
-                                                     int NG, int64_t pitch,
-                                                     __nv_bfloat16 *__restrict__ Ph,
-                                                     __nv_bfloat16 *__restrict__ Pl,
-                                                     __nv_bfloat16 *__restrict__ Qh,
-                                                     __nv_bfloat16 *__restrict__ Ql,
-                                                     __nv_bfloat16 *__restrict__ Th,
-                                                     __nv_bfloat16 *__restrict__ Tl,
+                                                     const float *__restrict__ y, int64_t n, int d, int dp,
+                                                     int NG, int64_t pitch, const uint32_t *__restrict__ mx,
+                                                     const float *__restrict__ c,
+                                                     uint16_t *__restrict__ Ph,
+                                                     uint16_t *__restrict__ Pl,
+                                                     uint16_t *__restrict__ Qh,
+                                                     uint16_t *__restrict__ Ql,
+                                                     uint16_t *__restrict__ Th,
+                                                     uint16_t *__restrict__ Tl,
                                                      float *__restrict__ a) {
     __shared__ float xs[32][97];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i0 = (int64_t)blockIdx.x * 32;
+    Scales q = {};
+    if (F16) q = scales_of(mx, d);
     for (int p = warp; p < 32; p += 8) {
         const int64_t i = i0 + p;
         if (i >= n) break;
         float acc = 0.f;
-        for (int t = lane; t < d; t += 32) {
-            const float xv = __ldg(x + i * d + t), yv = __ldg(y + i * d + t);
-            const float S = xv + yv, D = xv - yv;
-            const __nv_bfloat16 sh = __float2bfloat16_rn(S), dh = __float2bfloat16_rn(D);
-            const __nv_bfloat16 sl = __float2bfloat16_rn(S - __bfloat162float(sh));
-            const __nv_bfloat16 dl = __float2bfloat16_rn(D - __bfloat162float(dh));
-            const int64_t o = i * 2 * d + t;
-            Ph[o] = sh; Pl[o] = sl; Ph[o + d] = dh; Pl[o + d] = dl;
-            if (Qh) { Qh[o] = dh; Ql[o] = dl; Qh[o + d] = sh; Ql[o + d] = sl; }
+        for (int t = lane; t < dp; t += 32) {
+            const bool in = !F16 || t < d;
+            const float xv = in ? __ldg(x + i * d + t) : 0.f, yv = in ? __ldg(y + i * d + t) : 0.f;
+            const float ct = F16 && in ? __ldg(c + t) : 0.f;
+            const float S = F16 ? (xv - ct) + (yv - ct) : xv + yv, D = xv - yv;
+            uint16_t sh, sl, dh, dl;
+            if (F16) {
+                split_grid(S * q.s, sh, sl);
+                split_grid(D * q.d, dh, dl);
+            } else {
+                split_float<false>(S, sh, sl);
+                split_float<false>(D, dh, dl);
+            }
+            const int64_t o = i * 2 * dp + t;
+            Ph[o] = sh; Pl[o] = sl; Ph[o + dp] = dh; Pl[o + dp] = dl;
+            if (Qh) { Qh[o] = dh; Ql[o] = dl; Qh[o + dp] = sh; Ql[o + dp] = sl; }
             acc = fmaf(S, D, acc);
-            xs[p][t] = xv;
+            xs[p][t] = F16 ? xv - ct : xv;
         }
         acc = warp_sum_f32(acc);
         if (lane == 0) a[i] = acc;
@@ -909,16 +1146,14 @@ __global__ void __launch_bounds__(256) k_stress_prep(const float *__restrict__ x
             const int t = e >> 5, p = e & 31;
             const int64_t i = i0 + p;
             if (i >= n) continue;
-            const float v = t < d ? xs[p][t] : (t == d ? 1.0f : 0.0f);
-            const __nv_bfloat16 h = __float2bfloat16_rn(v);
-            Th[t * pitch + i] = h;
-            Tl[t * pitch + i] = __float2bfloat16_rn(v - __bfloat162float(h));
+            const float v = t < dp ? (F16 ? xs[p][t] * q.x : xs[p][t]) : (t == dp ? 1.0f : 0.0f);
+            split_float<F16>(v, Th[t * pitch + i], Tl[t * pitch + i]);
         }
     }
 }
 
 struct Layout {
-    int64_t Ph, Pl, Qh, Ql, Th, Tl, a, part, edm, deal, sums, total, pitch;
+    int64_t Ph, Pl, Qh, Ql, Th, Tl, a, part, edm, deal, sums, mx, total, pitch;
 };
 
 // The backward's chunks of the tile sequence: q per CTA, about kChunk
@@ -928,7 +1163,8 @@ static int64_t chunks_of(int64_t T, int64_t ctas) {
     return ctas * (q < 4 ? 4 : q);
 }
 
-static Layout layout_of(int64_t n, int64_t d, bool bwd) {
+// d: the operands' coordinates (f16: padded to a multiple of 32).
+static Layout layout_of(int64_t n, int64_t d, bool bwd, bool f16) {
     Layout L;
     const int64_t pq = align_up(n * 2 * d * 2, 1024);
     L.pitch = align_up(n, 8);
@@ -938,7 +1174,7 @@ static Layout layout_of(int64_t n, int64_t d, bool bwd) {
     L.a = L.Tl + xt;
     L.part = L.a + align_up(n * 4, 1024);
     L.edm = L.part + align_up(8 * (kMaxCtas + kReduceSlots), 1024);
-    L.deal = L.edm + ((!bwd && d % 64 == 0) ? edm_umma_workspace_bytes(n, d) : 0);
+    L.deal = L.edm + ((!bwd && !f16 && d % 64 == 0) ? edm_umma_workspace_bytes(n, d) : 0);
     // backward: the tile scan of the grid blocks (int each), the scan
     // blocks' offsets and the chunk starts (int64 each), for the largest
     // grid of any map and the most CTAs
@@ -955,26 +1191,29 @@ static Layout layout_of(int64_t n, int64_t d, bool bwd) {
                      align_up(8 * chunks_of(nb * (nb + 1) / 2, kMaxCtas), 1024);
     }
     L.sums = L.deal + deal_bytes;   // backward: the per-point sums S of the flushes
-    L.total = L.sums + (bwd ? align_up(4 * n, 1024) : 0);
+    L.mx = L.sums + (bwd ? align_up(4 * n, 1024) : 0);   // F16: the maxima and the centre
+    L.total = L.mx + (f16 ? 1024 : 0);
     return L;
 }
 
+template <bool F16>
 static cudaError_t optin_bwd() {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_stress_umma_bwd<MAP_LAMBDA>, a, SMEM_BYTES)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_stress_umma_bwd<MAP_BBOX>, a, SMEM_BYTES)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_stress_umma_bwd<MAP_RB>, a, SMEM_BYTES)) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_stress_umma_bwd<MAP_LINEAR>, a, SMEM_BYTES);
+    if ((e = cudaFuncSetAttribute(k_stress_umma_bwd<MAP_LAMBDA, F16>, a, SMEM_BYTES)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_stress_umma_bwd<MAP_BBOX, F16>, a, SMEM_BYTES)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_stress_umma_bwd<MAP_RB, F16>, a, SMEM_BYTES)) != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_stress_umma_bwd<MAP_LINEAR, F16>, a, SMEM_BYTES);
 }
 
+template <bool F16>
 static cudaError_t optin_fwd256() {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(f256::k_stress_umma_fwd<MAP_LAMBDA>, a, f256::SMEM2)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(f256::k_stress_umma_fwd<MAP_BBOX>, a, f256::SMEM2)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(f256::k_stress_umma_fwd<MAP_RB>, a, f256::SMEM2)) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(f256::k_stress_umma_fwd<MAP_LINEAR>, a, f256::SMEM2);
+    if ((e = cudaFuncSetAttribute(f256::k_stress_umma_fwd<MAP_LAMBDA, F16>, a, f256::SMEM2)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(f256::k_stress_umma_fwd<MAP_BBOX, F16>, a, f256::SMEM2)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(f256::k_stress_umma_fwd<MAP_RB, F16>, a, f256::SMEM2)) != cudaSuccess) return e;
+    return cudaFuncSetAttribute(f256::k_stress_umma_fwd<MAP_LINEAR, F16>, a, f256::SMEM2);
 }
 
 static int smem_optin() {
@@ -986,32 +1225,35 @@ static int smem_optin() {
     if (dev < 0 || dev >= 64) return SIMPLEX_EUNSUPPORTED;
     std::lock_guard<std::mutex> lk(mu);
     if (!done[dev]) {
-        if ((e = optin_fwd256()) != cudaSuccess || (e = optin_bwd()) != cudaSuccess)
+        if ((e = optin_fwd256<false>()) != cudaSuccess || (e = optin_bwd<false>()) != cudaSuccess ||
+            (e = optin_fwd256<true>()) != cudaSuccess || (e = optin_bwd<true>()) != cudaSuccess)
             return cuda_status(e);
         done[dev] = true;
     }
     return SIMPLEX_OK;
 }
 
+template <bool F16>
 static cudaError_t launch_bwd(int map, unsigned ctas, cudaStream_t s, const CUtensorMap *m, float *S,
                               const float *a, int64_t n, int d, int nb, int gx, int64_t T, int64_t nchunks,
-                              const int64_t *start, float scale4, float *grad, double *partials, int qshift) {
+                              const int64_t *start, float scale4, float *grad, double *partials, int qshift, int dg,
+                              const uint32_t *mx) {
     if (map == MAP_LAMBDA)
-        k_stress_umma_bwd<MAP_LAMBDA><<<ctas, kThreads, SMEM_BYTES, s>>>(
+        k_stress_umma_bwd<MAP_LAMBDA, F16><<<ctas, kThreads, SMEM_BYTES, s>>>(
             m[0], m[1], m[2], m[3], m[4], m[5], S, a, n, d, nb, gx, T, nchunks, start, scale4, grad,
-            partials, qshift);
+            partials, qshift, dg, mx);
     else if (map == MAP_BBOX)
-        k_stress_umma_bwd<MAP_BBOX><<<ctas, kThreads, SMEM_BYTES, s>>>(
+        k_stress_umma_bwd<MAP_BBOX, F16><<<ctas, kThreads, SMEM_BYTES, s>>>(
             m[0], m[1], m[2], m[3], m[4], m[5], S, a, n, d, nb, gx, T, nchunks, start, scale4, grad,
-            partials, qshift);
+            partials, qshift, dg, mx);
     else if (map == MAP_RB)
-        k_stress_umma_bwd<MAP_RB><<<ctas, kThreads, SMEM_BYTES, s>>>(
+        k_stress_umma_bwd<MAP_RB, F16><<<ctas, kThreads, SMEM_BYTES, s>>>(
             m[0], m[1], m[2], m[3], m[4], m[5], S, a, n, d, nb, gx, T, nchunks, start, scale4, grad,
-            partials, qshift);
+            partials, qshift, dg, mx);
     else
-        k_stress_umma_bwd<MAP_LINEAR><<<ctas, kThreads, SMEM_BYTES, s>>>(
+        k_stress_umma_bwd<MAP_LINEAR, F16><<<ctas, kThreads, SMEM_BYTES, s>>>(
             m[0], m[1], m[2], m[3], m[4], m[5], S, a, n, d, nb, gx, T, nchunks, start, scale4, grad,
-            partials, qshift);
+            partials, qshift, dg, mx);
     return cudaGetLastError();
 }
 
@@ -1034,9 +1276,10 @@ static cudaError_t chunk_starts(int map, int64_t total, int gx, int nb, int64_t 
 }
 
 // The forward runs as two-CTA clusters in 128 x 256 steps.
+template <bool F16>
 static cudaError_t launch_fwd(int map, unsigned ctas, cudaStream_t s, const CUtensorMap *m, const float *a,
                               int64_t n, int d, int nb, int nb2, int gx, int64_t total, double *partials,
-                              int qshift) {
+                              int qshift, int dg, const uint32_t *mx) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(kThreads);
@@ -1050,16 +1293,16 @@ static cudaError_t launch_fwd(int map, unsigned ctas, cudaStream_t s, const CUte
     cfg.attrs = at;
     cfg.numAttrs = 1;
     if (map == MAP_LAMBDA)
-        return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_LAMBDA>, m[0], m[1], m[2], m[3], a, n, d, nb,
-                                  nb2, gx, total, partials, qshift);
+        return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_LAMBDA, F16>, m[0], m[1], m[2], m[3], a, n, d, nb,
+                                  nb2, gx, total, partials, qshift, dg, mx);
     if (map == MAP_BBOX)
-        return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_BBOX>, m[0], m[1], m[2], m[3], a, n, d, nb,
-                                  nb2, gx, total, partials, qshift);
+        return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_BBOX, F16>, m[0], m[1], m[2], m[3], a, n, d, nb,
+                                  nb2, gx, total, partials, qshift, dg, mx);
     if (map == MAP_RB)
-        return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_RB>, m[0], m[1], m[2], m[3], a, n, d, nb,
-                                  nb2, gx, total, partials, qshift);
-    return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_LINEAR>, m[0], m[1], m[2], m[3], a, n, d, nb,
-                              nb2, gx, total, partials, qshift);
+        return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_RB, F16>, m[0], m[1], m[2], m[3], a, n, d, nb,
+                                  nb2, gx, total, partials, qshift, dg, mx);
+    return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_LINEAR, F16>, m[0], m[1], m[2], m[3], a, n, d, nb,
+                              nb2, gx, total, partials, qshift, dg, mx);
 }
 
 // Two-CTA clusters of the forward kernel that fit on the device at once (one
@@ -1083,7 +1326,7 @@ static int64_t max_pairs(int sms) {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int num = 0;
-        if (cudaOccupancyMaxActiveClusters(&num, f256::k_stress_umma_fwd<MAP_LAMBDA>, &cfg) != cudaSuccess ||
+        if (cudaOccupancyMaxActiveClusters(&num, f256::k_stress_umma_fwd<MAP_LAMBDA, false>, &cfg) != cudaSuccess ||
             num < 1) {
             cudaGetLastError();
             num = sms / 2;
@@ -1102,42 +1345,61 @@ bool stress_use_umma(int64_t d, int prec) {
 }
 
 int64_t stress_umma_workspace_bytes(int64_t n, int64_t d, bool bwd) {
-    return 1024 + summa::layout_of(n, d, bwd).total;
+    return 1024 + summa::layout_of(n, d, bwd, false).total;
 }
 
-int stress_umma_run(bool bwd, int64_t n, int64_t d, const float *x, const float *y, float *d_out,
-                    double *loss, double gscale, float *grad, int map, void *ws, int64_t ws_bytes,
-                    cudaStream_t s) {
+static int64_t padded(int64_t d) { return (d + 31) / 32 * 32; }
+
+// Both paths measured: the launches before the main kernel (centre, maxima,
+// operands; the backward's tile scan) cost the F16 path 37 us forward and 58 us
+// backward at any size, the FP32 kernels grow with n^2 (d + 20):
+//   forward   n = 2561, d = 64: 41 against 53 us; 4096, 5: 36 and 42;
+//             2560, 20: 38 and 30; 3000, 3: 39 and 29
+//   backward  n = 2560, d = 20: 60 against 66 us; 3000, 3: 54 and 76;
+//             2048, 33: 60 and 57; 2560, 2: 58 and 59
+// n = 10000, d = 64: 78 against 575 us forward, 175 against 1125 us backward;
+// n = 20000, d = 96: 0.26 against 3.35 ms, 0.66 against 7.80 ms.
+bool stress_f16_ok(int64_t n, int64_t d, bool bwd) {
+    if (d > summa::kMaxDim || n < 1024) return false;
+    return (double)n * (double)n * (double)(d + 20) >= (bwd ? 2.0e8 : 3.6e8);
+}
+
+int64_t stress_f16_workspace_bytes(int64_t n, int64_t d, bool bwd) {
+    return 1024 + summa::layout_of(n, padded(d), bwd, true).total;
+}
+
+// d: coordinates in x, y and grad; dp: in the operands.
+template <bool F16>
+static int run(bool bwd, int64_t n, int64_t d, int64_t dp, const float *x, const float *y, double *loss, double gscale,
+               float *grad, int map, void *ws, cudaStream_t s) {
     using namespace summa;
-    if (!stress_umma_ok(d)) return SIMPLEX_EUNSUPPORTED;
-    if (!aligned(x, 16)) return SIMPLEX_EALIGN;
-    if (!ws || ws_bytes < stress_umma_workspace_bytes(n, d, bwd) || !aligned(ws, 256))
-        return SIMPLEX_EWORKSPACE;
     const int64_t nb = (n + TM - 1) / TM;
     const Grid g = grid2(nb, map);
     if (!grid_fits(g)) return SIMPLEX_EOVERFLOW;
-    const Layout L = layout_of(n, d, bwd);
+    const Layout L = layout_of(n, dp, bwd, F16);
     unsigned char *w = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(ws) + 1023) & ~uintptr_t(1023));
-    auto bf = [&](int64_t off) { return reinterpret_cast<__nv_bfloat16 *>(w + off); };
+    auto bf = [&](int64_t off) { return reinterpret_cast<uint16_t *>(w + off); };
     float *a = reinterpret_cast<float *>(w + L.a);
     double *partials = reinterpret_cast<double *>(w + L.part);
-    const int NG = (int)d + 16;
-    // Q = [Delta | S] is P = [S | Delta] with its two halves swapped: where d
+    uint32_t *mx = F16 ? reinterpret_cast<uint32_t *>(w + L.mx) : nullptr;
+    float *c = F16 ? reinterpret_cast<float *>(w + L.mx + 16) : nullptr;
+    const int NG = (int)dp + 16;
+    // Q = [Delta | S] is P = [S | Delta] with its two halves swapped: where dp
     // is a multiple of the K chunk, Q's chunk c is P's chunk at column
-    // (64 c + d) mod 2d, so the kernels read Q's tiles from P's memory (one
+    // (64 c + dp) mod 2 dp, so the kernels read Q's tiles from P's memory (one
     // operand copy fewer to write and to keep in L2); otherwise Q is written.
-    const bool qview = d % KC == 0;
-    const int qshift = qview ? (int)d : 0;
-    CUtensorMap m[6];
-    if (!make_map_bf16(&m[0], bf(L.Ph), n, 2 * d, 2 * d, TM) ||
-        !make_map_bf16(&m[1], bf(L.Pl), n, 2 * d, 2 * d, TM))
+    const bool qview = dp % KC == 0;
+    const int qshift = qview ? (int)dp : 0;
+    CUtensorMap m[6];   // (16-bit elements: the maps only copy them)
+    if (!make_map_bf16(&m[0], bf(L.Ph), n, 2 * dp, 2 * dp, TM) ||
+        !make_map_bf16(&m[1], bf(L.Pl), n, 2 * dp, 2 * dp, TM))
         return SIMPLEX_ECUDA;
     if (qview) {
         m[2] = m[0];
         m[3] = m[1];
-    } else if (!make_map_bf16(&m[2], bf(L.Qh), n, 2 * d, 2 * d, TM) ||
-               !make_map_bf16(&m[3], bf(L.Ql), n, 2 * d, 2 * d, TM)) {
+    } else if (!make_map_bf16(&m[2], bf(L.Qh), n, 2 * dp, 2 * dp, TM) ||
+               !make_map_bf16(&m[3], bf(L.Ql), n, 2 * dp, 2 * dp, TM)) {
         return SIMPLEX_ECUDA;
     }
     if (bwd) {
@@ -1150,14 +1412,23 @@ int stress_umma_run(bool bwd, int64_t n, int64_t d, const float *x, const float 
     }
     int st = smem_optin();
     if (st) return st;
-    k_stress_prep<<<(unsigned)((n + 31) / 32), 256, 0, s>>>(
-        x, y, n, (int)d, NG, L.pitch, bf(L.Ph), bf(L.Pl), qview ? nullptr : bf(L.Qh), qview ? nullptr : bf(L.Ql),
-        bwd ? bf(L.Th) : nullptr, bwd ? bf(L.Tl) : nullptr, a);
-    note_launches(1);
-    if ((st = launch_status())) return st;
     int dev = 0, sms = 0;
     if ((st = cuda_status(cudaGetDevice(&dev)))) return st;
     if ((st = cuda_status(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))) return st;
+    if (F16) {
+        k_stress_centre<<<1, 8 * kMaxDim, 0, s>>>(x, n, (int)d, c, mx);
+        note_launches(1);
+        if ((st = launch_status())) return st;
+        const int64_t mb = (n * d + 1023) / 1024;   // four elements a thread, at most two blocks an SM
+        k_stress_max<<<(unsigned)(mb < 2 * sms ? mb : 2 * sms), 256, 0, s>>>(x, y, n * d, (int)d, c, mx);
+        note_launches(1);
+        if ((st = launch_status())) return st;
+    }
+    k_stress_prep<F16><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(
+        x, y, n, (int)d, (int)dp, NG, L.pitch, mx, c, bf(L.Ph), bf(L.Pl), qview ? nullptr : bf(L.Qh),
+        qview ? nullptr : bf(L.Ql), bwd ? bf(L.Th) : nullptr, bwd ? bf(L.Tl) : nullptr, a);
+    note_launches(1);
+    if ((st = launch_status())) return st;
     int64_t ctas;
     cudaError_t le;
     if (bwd) {
@@ -1176,8 +1447,8 @@ int stress_umma_run(bool bwd, int64_t n, int64_t d, const float *x, const float 
         if ((st = cuda_status(cudaMemsetAsync(grad, 0, sizeof(float) * (size_t)(n * d), s)))) return st;
         if ((st = cuda_status(cudaMemsetAsync(S, 0, sizeof(float) * (size_t)n, s)))) return st;
         prof_begin(s);
-        le = launch_bwd(map, (unsigned)ctas, s, m, S, a, n, (int)d, (int)nb, (int)g.gx, T, nchunks, start,
-                        (float)(4.0 * gscale), grad, loss ? partials : nullptr, qshift);
+        le = launch_bwd<F16>(map, (unsigned)ctas, s, m, S, a, n, (int)dp, (int)nb, (int)g.gx, T, nchunks, start,
+                             (float)(4.0 * gscale), grad, loss ? partials : nullptr, qshift, (int)d, mx);
     } else {
         // two-CTA clusters over the map's grid of 256 x 256 super-blocks
         const int64_t nb2 = (nb + 1) / 2;
@@ -1189,28 +1460,48 @@ int stress_umma_run(bool bwd, int64_t n, int64_t d, const float *x, const float 
         if (clusters > kMaxCtas / 2) clusters = kMaxCtas / 2;
         ctas = 2 * clusters;
         prof_begin(s);
-        le = launch_fwd(map, (unsigned)ctas, s, m, a, n, (int)d, (int)nb, (int)nb2, (int)g2.gx, total2,
-                        partials, qshift);
+        le = launch_fwd<F16>(map, (unsigned)ctas, s, m, a, n, (int)dp, (int)nb, (int)nb2, (int)g2.gx, total2,
+                             partials, qshift, (int)d, mx);
     }
     prof_end(s);
     note_launches(1);
     if (le != cudaSuccess) return cuda_status(le);
     if ((st = launch_status())) return st;
-    if (bwd) {
+    if (!bwd) return reduce_partials(partials, ctas, partials + kMaxCtas, loss, s);
+    const float *S = reinterpret_cast<const float *>(w + L.sums);
+    if (F16) {
+        k_stress_sx_centred<<<(unsigned)((n * d + 255) / 256), 256, 0, s>>>(x, c, S, n, (int)d, (float)(4.0 * gscale), grad);
+    } else {
         const int64_t f4 = n * d / 4;
-        k_stress_sx<<<(unsigned)((f4 + 255) / 256), 256, 0, s>>>(x, reinterpret_cast<const float *>(w + L.sums), n,
-                                                              (int)d, (float)(4.0 * gscale), grad);
-        note_launches(1);
-        if ((st = launch_status())) return st;
-        return loss ? reduce_partials(partials, ctas, partials + kMaxCtas, loss, s) : SIMPLEX_OK;
+        k_stress_sx<<<(unsigned)((f4 + 255) / 256), 256, 0, s>>>(x, S, n, (int)d, (float)(4.0 * gscale), grad);
     }
-    if ((st = reduce_partials(partials, ctas, partials + kMaxCtas, loss, s))) return st;
-    if (!d_out) return SIMPLEX_OK;
+    note_launches(1);
+    if ((st = launch_status())) return st;
+    return loss ? reduce_partials(partials, ctas, partials + kMaxCtas, loss, s) : SIMPLEX_OK;
+}
+
+int stress_umma_run(bool bwd, int64_t n, int64_t d, const float *x, const float *y, float *d_out,
+                    double *loss, double gscale, float *grad, int map, void *ws, int64_t ws_bytes,
+                    cudaStream_t s) {
+    using namespace summa;
+    if (!stress_umma_ok(d)) return SIMPLEX_EUNSUPPORTED;
+    if (!aligned(x, 16)) return SIMPLEX_EALIGN;
+    if (!ws || ws_bytes < stress_umma_workspace_bytes(n, d, bwd) || !aligned(ws, 256))
+        return SIMPLEX_EWORKSPACE;
+    const int st = run<false>(bwd, n, d, d, x, y, loss, gscale, grad, map, ws, s);
+    if (st || !d_out) return st;
     // the packed D itself: tensor-core EDM where it applies, else FP32
+    unsigned char *w = reinterpret_cast<unsigned char *>(
+        (reinterpret_cast<uintptr_t>(ws) + 1023) & ~uintptr_t(1023));
     if (d % 64 == 0)
-        return simplex_edm_packed(n, d, x, d_out, map, SIMPLEX_PREC_BF16X3, w + L.edm,
+        return simplex_edm_packed(n, d, x, d_out, map, SIMPLEX_PREC_BF16X3, w + layout_of(n, d, bwd, false).edm,
                                   edm_umma_workspace_bytes(n, d), s);
     return simplex_edm_packed(n, d, x, d_out, map, SIMPLEX_PREC_FP32, nullptr, 0, s);
+}
+
+int stress_f16_run(bool bwd, int64_t n, int64_t d, const float *x, const float *y, double *loss, double gscale,
+                   float *grad, int map, void *ws, cudaStream_t s) {
+    return run<true>(bwd, n, d, padded(d), x, y, loss, gscale, grad, map, ws, s);
 }
 
 int stress_umma_errors(cudaStream_t s) {

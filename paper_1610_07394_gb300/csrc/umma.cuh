@@ -27,9 +27,9 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n, bool a_mn_major,
            ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// The same with A = B = FP16 (format 0 in bits 7-9 and 10-12), both K-major.
-__host__ __device__ constexpr uint32_t idesc_f16(int m, int n) {
-    return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+// The same with A = B = FP16 (format 0 in bits 7-9 and 10-12).
+__host__ __device__ constexpr uint32_t idesc_f16(int m, int n, bool a_mn_major = false, bool b_mn_major = false) {
+    return idesc_bf16(m, n, a_mn_major, b_mn_major) & ~((1u << 7) | (1u << 10));
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -202,6 +202,47 @@ __device__ __forceinline__ void mma_bf16x3_w(uint32_t tmem_d, uint64_t ah, uint6
         "@e tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %4, %5, t;\n\t"
         "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %3, %5, t;\n\t}" ::"r"(tmem_d),
         "l"(ah), "l"(al), "l"(bh), "l"(bl), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// The four products of a hi + lo step into two accumulators, D0 (+)= Ah Bh and
+// D1 (+)= Ah Bl + Al Bh + Al Bl (see mma_bf16x3_w).
+__device__ __forceinline__ void mma_split4_w(uint32_t d0, uint32_t d1, uint64_t ah, uint64_t al, uint64_t bh,
+                                             uint64_t bl, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, e, t;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %7, 0;\n\t"
+        "setp.eq.b32 t, %7, %7;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %2, %4, %6, p;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%1], %2, %5, %6, p;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%1], %3, %4, %6, t;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%1], %3, %5, %6, t;\n\t}" ::"r"(d0),
+        "r"(d1), "l"(ah), "l"(al), "l"(bh), "l"(bl), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// The cross products alone, D (+)= Ah Bl + Al Bh, and one product D += A B.
+__device__ __forceinline__ void mma_cross_w(uint32_t tmem_d, uint64_t ah, uint64_t al, uint64_t bh, uint64_t bl,
+                                            uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, e, t;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.eq.b32 t, %6, %6;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %4, %5, p;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %3, %5, t;\n\t}" ::"r"(tmem_d),
+        "l"(ah), "l"(al), "l"(bh), "l"(bl), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_add_w(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred e, t;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.eq.b32 t, %3, %3;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, t;\n\t}" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc)
         : "memory");
 }
 
@@ -484,6 +525,11 @@ using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t,
                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 inline EncodeTiled encode_fn() {
+    // The driver's call needs the device's context current on this thread; a
+    // thread that has made no runtime call that binds it yet (an autograd
+    // worker whose tensors came from a cache) gets it here.
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return nullptr;
     static std::once_flag once;
     static EncodeTiled fn = nullptr;
     std::call_once(once, [] {
