@@ -18,6 +18,7 @@ backward passes call the library's adjoint kernels.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 
 import torch
@@ -114,7 +115,9 @@ def _prec(p) -> int:
 
 def _stream(stream=None) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        # torch.cuda.current_stream().cuda_stream without the Stream object
+        # (2 us of a small call's host time)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -149,6 +152,11 @@ def simplex_grid_blocks(m: int, nb: int, map="lambda") -> int:
 def simplex_workspace_bytes(op, n: int, d: int, map="lambda", prec="fp32") -> int:
     return lib().simplex_workspace_bytes(OPS[op] if isinstance(op, str) else op, n, d,
                                          _map(map), _prec(prec))
+
+
+# The size depends on these arguments alone; the wrappers below ask for it on
+# every call.
+_workspace_bytes = functools.lru_cache(maxsize=1024)(simplex_workspace_bytes)
 
 
 def simplex_map_blocks(m: int, nb: int, map, out: torch.Tensor, stream=None):
@@ -274,7 +282,7 @@ def simplex_profile_read():
 
 def workspace(op, n: int, d: int, map="lambda", prec="fp32", device="cuda") -> torch.Tensor | None:
     """A workspace buffer of the size the library asks for (None if none)."""
-    b = simplex_workspace_bytes(op, n, d, map, prec)
+    b = _workspace_bytes(op, n, d, map, prec)
     if b < 0:
         raise ValueError("bad arguments for workspace sizing")
     return torch.empty(b, dtype=torch.uint8, device=device) if b else None
