@@ -241,7 +241,7 @@ int64_t simplex_edm_tiles_len(int64_t n);
  * the denominator (cosines from the law of cosines on unsoftened squares).
  * d must be 3.  x: device, n*3 FP32.  energy: device, 1 double (written).
  * Per-triple arithmetic is FP32; the reduction across blocks is FP64.
- * From 1664 points (up to the table limit) the sum runs as contractions of
+ * From 1280 points (up to the table limit) the sum runs as contractions of
  * pair matrices on the tensor cores, FP16 hi + lo splits of FP32 terms with
  * FP32 sums, over 256 x 256 super-blocks of pairs that the map's 2-simplex
  * grid lists, and the triples of each point's nearest neighbour one by one in

@@ -16,10 +16,10 @@
 // packed FP32 loop (atm.cu) spends 12 (energy) or 32 (forces) operations per
 // two triples on the FMA pipe, which bounds it at 65-70% of its issue rate
 // with the tensor cores idle.  Energy and forces, before and after:
-// n = 1024 297 -> 157 us, n = 3000 6.47 -> 1.59 ms, n = 4096 15.4 -> 3.75 ms,
+// n = 1024 297 -> 152 us, n = 3000 6.47 -> 1.56 ms, n = 4096 15.4 -> 3.77 ms,
 // n = 16384 960 -> 240 ms (1390 TFLOP/s of FP16 products, the tensor pipe 85%
 // busy at the 1.64 GHz that the power limit leaves); energy alone
-// n = 3000 2.18 -> 0.89 ms, n = 4096 5.16 -> 1.81 ms.
+// n = 3000 2.18 -> 0.85 ms, n = 4096 5.16 -> 1.69 ms.
 //
 // Near pairs.  Each point's pair with its nearest neighbour is left out of the
 // matrices, and the n^2 triples that hold such a pair are evaluated one by one
@@ -127,8 +127,12 @@ inline int64_t tile_sets(const Table &T) {
 // column inside a strip, so that the clusters at work at one time share few
 // row and column blocks (each k chunk's tiles are then read from HBM once
 // for many clusters).
+// Row by row instead (`rows`) for the energy while its operands fit the L2
+// cache (n <= 6144): its chunks shrink with Y, so that list is sorted by length,
+// which the back-and-forth dealing needs to fill the clusters evenly.
 constexpr int kStrip = 8;
-__host__ __device__ __forceinline__ int super_rank(int X, int Y, int ns) {
+__host__ __device__ __forceinline__ int super_rank(int X, int Y, int ns, bool rows) {
+    if (rows) return Y * (Y + 1) / 2 + X;
     const int r0 = Y / kStrip * kStrip;
     const int h = ns - r0 < kStrip ? ns - r0 : kStrip;
     const int base = r0 * (r0 + 1) / 2;
@@ -262,7 +266,8 @@ struct Walk {
 // grid blocks to the list of super-blocks.
 template <int MAP>
 __global__ void __launch_bounds__(256) k_atm_prep(int64_t n, const float *__restrict__ x, float eps, int ns,
-                                                  int gx, int cells, float *__restrict__ uinv, int *__restrict__ nn,
+                                                  int gx, int cells, bool rows, float *__restrict__ uinv,
+                                                  int *__restrict__ nn,
                                                   int *__restrict__ list, double *__restrict__ near_energy,
                                                   double *__restrict__ forces) {
     const int lane = threadIdx.x & 31;
@@ -271,8 +276,8 @@ __global__ void __launch_bounds__(256) k_atm_prep(int64_t n, const float *__rest
     if (gt < cells) {
         const int wy = (int)(gt / gx), wx = (int)(gt - (int64_t)wy * gx);
         const List2 L = decode2<MAP>((uint32_t)wx, (uint32_t)wy, ns);
-        if (L.cnt > 0) list[super_rank(L.x[0], L.y[0], ns)] = L.x[0] | (L.y[0] << 16);
-        if (L.cnt > 1) list[super_rank(L.x[1], L.y[1], ns)] = L.x[1] | (L.y[1] << 16);
+        if (L.cnt > 0) list[super_rank(L.x[0], L.y[0], ns, rows)] = L.x[0] | (L.y[0] << 16);
+        if (L.cnt > 1) list[super_rank(L.x[1], L.y[1], ns, rows)] = L.x[1] | (L.y[1] << 16);
     }
     const int64_t i = gt >> 5;
     if (i >= n) return;
@@ -468,7 +473,7 @@ __global__ void __launch_bounds__(kNearThreads) k_atm_near(int64_t n, const floa
     float ax, ay, az, ra, Ra;   // a = x_i - x_j
     unit_of(xi - xj, yi - yj, zi - zj, eps, ax, ay, az, ra, Ra);
     // 2nd neighbours' R of the two points (their scales hold its exponent)
-    const float big = active ? 0x1p24f * __ldg(uinv + i) * __ldg(uinv + j) : 0.f;
+    const float big = active ? 0x1p26f * __ldg(uinv + i) * __ldg(uinv + j) : 0.f;
     float eh = 0.f, el = 0.f, fh[6] = {}, fl[6] = {};
     for (int q0 = 0; q0 < kn; q0 += 16) {
         float es = 0.f, fs[6] = {};
@@ -1085,10 +1090,11 @@ static int energy_passes(int64_t n, int64_t tab_bytes, int *cut) {
 
 // The contraction's fixed work (one 256 x 256 super-block per 256 points, six or
 // seven launches) pays from 640 points for the forces (n = 512: 88 against
-// 67 us, 600: 110 and 109, 700: 122 and 135, 1024: 157 and 298) and, as its
-// tables take two or three passes through the energy's smaller workspace,
-// from 1664 for the energy (n = 1536: 345 against 327 us, 2048: 438 and 690).
-static constexpr int64_t kMinForces = 640, kMinEnergy = 1664;
+// 67 us, 640: 103 and 116, 1024: 152 and 297) and, as its tables take two or
+// three passes through the energy's smaller workspace, from 1280 for the energy
+// (n = 1024: 131 against 106 us, 1152: 224 and 175, 1280: 191 and 214, 1536:
+// 224 and 326, 2048: 343 and 690).
+static constexpr int64_t kMinForces = 640, kMinEnergy = 1280;
 
 bool atm_umma_forces_ok(int64_t n, int64_t tab_bytes, int64_t rest_bytes) {
     using namespace aumma;
@@ -1123,11 +1129,12 @@ int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float ep
     if ((st = smem_optin(clusters))) return st;
     const unsigned pb = (unsigned)((n + 7) / 8);
     double *fz = want_forces ? forces : nullptr;
-    if (map == MAP_LAMBDA) k_atm_prep<MAP_LAMBDA><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, uinv, nn, list, near_energy, fz);
-    else if (map == MAP_BBOX) k_atm_prep<MAP_BBOX><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, uinv, nn, list, near_energy, fz);
-    else k_atm_prep<MAP_LINEAR><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, uinv, nn, list, near_energy, fz);
+    const bool rows = !want_forces && ns <= 24;
+    if (map == MAP_LAMBDA) k_atm_prep<MAP_LAMBDA><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, fz);
+    else if (map == MAP_BBOX) k_atm_prep<MAP_BBOX><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, fz);
+    else k_atm_prep<MAP_LINEAR><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, fz);
     // near pairs: 128 pairs by `seg` points per block, enough blocks for the chip
-    const int seg = n < 4096 ? 32 : 128;
+    const int seg = n < 2048 ? 16 : n < 4096 ? 32 : 128;
     const dim3 ng((unsigned)((n + kNearThreads - 1) / kNearThreads), (unsigned)((n + seg - 1) / seg));
     if (want_forces) k_atm_near<true><<<ng, kNearThreads, 0, s>>>(n, x, nu, eps, seg, uinv, nn, energy ? near_energy : nullptr, forces);
     else k_atm_near<false><<<ng, kNearThreads, 0, s>>>(n, x, nu, eps, seg, uinv, nn, near_energy, nullptr);
@@ -1138,7 +1145,7 @@ int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float ep
     // products per segment of the six-product outputs: long segments save
     // epilogues, short ones fill the clusters
     const int64_t per = (int64_t)S * 25 / clusters;   // products per cluster
-    const int G = want_forces ? (per >= 12 ? 6 : per >= 3 ? 3 : 1) : (per >= 40 ? 6 : per >= 20 ? 3 : 1);
+    const int G = want_forces ? (per >= 12 ? 6 : per >= 3 ? 3 : 1) : (per >= 10 ? 3 : 2);
     const int64_t segs = (int64_t)S * (3 * (6 / G) + 7);
     if (clusters > segs) clusters = (int)segs;
     for (int p = 0; p < passes; ++p) {

@@ -205,6 +205,60 @@ __global__ void __launch_bounds__(256) k_chunk_starts(int64_t total, int64_t nbl
     start[c] = 2 * a + (rr - loc[a]);
 }
 
+// The three steps in one block, for grids of at most kOneScan blocks (three
+// launches cost more than the scan there): the counts of 1024 grid blocks at
+// a time scanned with a running total, then every chunk's first tile by a
+// binary search over the whole prefix (in loc).
+constexpr int64_t kOneScan = 16384;
+
+template <int MAP>
+__global__ void __launch_bounds__(1024) k_chunk_starts_small(int total, int gx, int nb, int64_t T, int64_t N,
+                                                             int *__restrict__ loc, int64_t *__restrict__ start) {
+    __shared__ int wsum[32];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    int carry = 0;
+    for (int base = 0; base < total; base += 1024) {
+        const int w = base + (int)threadIdx.x;
+        int c = 0;
+        if (w < total) {
+            const int wy = w / gx;
+            c = decode_grid2<MAP>(w, w - wy * gx, wy, nb).cnt;
+        }
+        int v = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += u;
+        }
+        if (lane == 31) wsum[wp] = v;
+        __syncthreads();
+        if (wp == 0) {
+            int t = wsum[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, t, o);
+                if (lane >= o) t += u;
+            }
+            wsum[lane] = t;
+        }
+        __syncthreads();
+        if (w < total) loc[w] = carry + (wp ? wsum[wp - 1] : 0) + v - c;
+        carry += wsum[31];
+        __syncthreads();
+    }
+    __threadfence_block();
+    __syncthreads();
+    for (int64_t c = threadIdx.x; c < N; c += 1024) {
+        const int64_t r = c * T / N;
+        int a = 0, z = total - 1;
+        while (a < z) {
+            const int mid = (a + z + 1) >> 1;
+            if (loc[mid] <= r) a = mid; else z = mid - 1;
+        }
+        start[c] = 2 * (int64_t)a + (r - loc[a]);
+    }
+}
+
 template <int MAP>
 struct ChunkWalk {
     const int64_t *start;
@@ -1108,12 +1162,18 @@ __global__ void __launch_bounds__(256) k_stress_prep(const float *__restrict__ x
                                                      uint16_t *__restrict__ Ql,
                                                      uint16_t *__restrict__ Th,
                                                      uint16_t *__restrict__ Tl,
-                                                     float *__restrict__ a) {
+                                                     float *__restrict__ a, float *__restrict__ grad,
+                                                     float *__restrict__ S_) {
     __shared__ float xs[32][97];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i0 = (int64_t)blockIdx.x * 32;
     Scales q = {};
     if (F16) q = scales_of(mx, d);
+    if (Th) {   // the backward adds into these
+        const int64_t e0 = i0 * d, e1 = (i0 + 32 < n ? i0 + 32 : n) * d;
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) grad[e] = 0.f;
+        if (threadIdx.x < 32 && i0 + threadIdx.x < n) S_[i0 + threadIdx.x] = 0.f;
+    }
     for (int p = warp; p < 32; p += 8) {
         const int64_t i = i0 + p;
         if (i >= n) break;
@@ -1261,8 +1321,18 @@ static cudaError_t launch_bwd(int map, unsigned ctas, cudaStream_t s, const CUte
 // tile of every chunk, into the workspace.
 static cudaError_t chunk_starts(int map, int64_t total, int gx, int nb, int64_t T, int64_t nchunks, int *loc,
                                 int64_t *boff, int64_t *start, cudaStream_t s) {
+    if (total <= kOneScan) {
+        const int t = (int)total;
+        if (map == MAP_LAMBDA) k_chunk_starts_small<MAP_LAMBDA><<<1, 1024, 0, s>>>(t, gx, nb, T, nchunks, loc, start);
+        else if (map == MAP_BBOX) k_chunk_starts_small<MAP_BBOX><<<1, 1024, 0, s>>>(t, gx, nb, T, nchunks, loc, start);
+        else if (map == MAP_RB) k_chunk_starts_small<MAP_RB><<<1, 1024, 0, s>>>(t, gx, nb, T, nchunks, loc, start);
+        else k_chunk_starts_small<MAP_LINEAR><<<1, 1024, 0, s>>>(t, gx, nb, T, nchunks, loc, start);
+        note_launches(1);
+        return cudaGetLastError();
+    }
     const int64_t nblk = (total + kScanBlock - 1) / kScanBlock;
     const unsigned b = (unsigned)nblk;
+    note_launches(3);
     if (map == MAP_LAMBDA) k_tile_scan<MAP_LAMBDA><<<b, kScanBlock, 0, s>>>(total, gx, nb, loc, boff);
     else if (map == MAP_BBOX) k_tile_scan<MAP_BBOX><<<b, kScanBlock, 0, s>>>(total, gx, nb, loc, boff);
     else if (map == MAP_RB) k_tile_scan<MAP_RB><<<b, kScanBlock, 0, s>>>(total, gx, nb, loc, boff);
@@ -1426,7 +1496,8 @@ static int run(bool bwd, int64_t n, int64_t d, int64_t dp, const float *x, const
     }
     k_stress_prep<F16><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(
         x, y, n, (int)d, (int)dp, NG, L.pitch, mx, c, bf(L.Ph), bf(L.Pl), qview ? nullptr : bf(L.Qh),
-        qview ? nullptr : bf(L.Ql), bwd ? bf(L.Th) : nullptr, bwd ? bf(L.Tl) : nullptr, a);
+        qview ? nullptr : bf(L.Ql), bwd ? bf(L.Th) : nullptr, bwd ? bf(L.Tl) : nullptr, a, grad,
+        reinterpret_cast<float *>(w + L.sums));
     note_launches(1);
     if ((st = launch_status())) return st;
     int64_t ctas;
@@ -1442,10 +1513,7 @@ static int run(bool bwd, int64_t n, int64_t d, int64_t dp, const float *x, const
         int64_t *start = reinterpret_cast<int64_t *>(reinterpret_cast<unsigned char *>(boff) + align_up(8 * nblk, 1024));
         if ((st = cuda_status(chunk_starts(map, total, (int)g.gx, (int)nb, T, nchunks, loc, boff, start, s))))
             return st;
-        note_launches(3);
         float *S = reinterpret_cast<float *>(w + L.sums);
-        if ((st = cuda_status(cudaMemsetAsync(grad, 0, sizeof(float) * (size_t)(n * d), s)))) return st;
-        if ((st = cuda_status(cudaMemsetAsync(S, 0, sizeof(float) * (size_t)n, s)))) return st;
         prof_begin(s);
         le = launch_bwd<F16>(map, (unsigned)ctas, s, m, S, a, n, (int)dp, (int)nb, (int)g.gx, T, nchunks, start,
                              (float)(4.0 * gscale), grad, loss ? partials : nullptr, qshift, (int)d, mx);

@@ -525,11 +525,6 @@ using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t,
                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 inline EncodeTiled encode_fn() {
-    // The driver's call needs the device's context current on this thread; a
-    // thread that has made no runtime call that binds it yet (an autograd
-    // worker whose tensors came from a cache) gets it here.
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return nullptr;
     static std::once_flag once;
     static EncodeTiled fn = nullptr;
     std::call_once(once, [] {
@@ -543,63 +538,67 @@ inline EncodeTiled encode_fn() {
     return fn;
 }
 
+// The driver's call needs the device's context current on this thread; a
+// thread that has made no runtime call that binds it yet (an autograd worker
+// whose tensors came from a cache) gets it on the first failure.
+template <typename... Args>
+inline bool encode_tiled(Args... args) {
+    EncodeTiled f = encode_fn();
+    if (!f) return false;
+    if (f(args...) == CUDA_SUCCESS) return true;
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess && f(args...) == CUDA_SUCCESS;
+}
+
 // A rows x cols BF16 matrix with row pitch `pitch` elements (pitch * 2 a
 // multiple of 16 bytes, base 16-byte aligned), boxes of box_rows rows x 64
 // columns (128 bytes: one swizzle row), 128-byte swizzle, zero fill outside.
 inline bool make_map_bf16(CUtensorMap *m, void *ptr, int64_t rows, int64_t cols, int64_t pitch,
                           int box_rows) {
-    EncodeTiled f = encode_fn();
-    if (!f) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)pitch * 2};
     const cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
-    return f(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box, estr,
+    return encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // `rows` rows of 64 16-bit elements (128 bytes, base 16-byte aligned), boxes
 // of box_rows whole rows, copied as they lie (no swizzle).
 inline bool make_map_rows16(CUtensorMap *m, void *ptr, int64_t rows, int box_rows) {
-    EncodeTiled f = encode_fn();
-    if (!f) return false;
     const cuuint64_t dims[2] = {64u, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {128u};
     const cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
-    return f(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ptr, dims, strides, box, estr,
+    return encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ptr, dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // The map of make_map_bf16 with boxes of 32 BF16 (64 bytes) per row in the 64-byte swizzle.
 inline bool make_map_bf16_sw64(CUtensorMap *m, void *ptr, int64_t rows, int64_t cols, int64_t pitch,
                                int box_rows) {
-    EncodeTiled f = encode_fn();
-    if (!f) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)pitch * 2};
     const cuuint32_t box[2] = {32u, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
-    return f(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box, estr,
+    return encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // The tile-packed EDM output as a 3-D FP32 tensor [tiles][128 rows][128
 // columns] (base 16-byte aligned), boxes of 32 columns x 32 rows of one tile
 // (4 KB, one 128-byte swizzle row per tile row), 128-byte swizzle.
 inline bool make_map_tiles_f32(CUtensorMap *m, float *out, int64_t tiles) {
-    EncodeTiled f = encode_fn();
-    if (!f) return false;
     const cuuint64_t dims[3] = {128u, 128u, (cuuint64_t)tiles};
     const cuuint64_t strides[2] = {128u * 4u, 128u * 128u * 4u};
     const cuuint32_t box[3] = {32u, 32u, 1u};
     const cuuint32_t estr[3] = {1, 1, 1};
-    return f(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, out, dims, strides, box, estr,
+    return encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, out, dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // Shared-memory byte offset of float4 chunk c (0..7) of row r (0..31) inside a

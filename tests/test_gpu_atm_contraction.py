@@ -1,5 +1,5 @@
 """ATM energy and forces where they run as contractions on the tensor cores
-(forces from 640 points, energy from 1664), at the edges of its tiles (128 rows,
+(forces from 640 points, energy from 1280), at the edges of its tiles (128 rows,
 256-row super-blocks, 64-point chunks) against the FP64 oracle, with the
 tolerances of the FP32 path: energy 1e-6, forces 1e-4 per atom and, for clouds
 of close pairs, 32 u kappa per atom."""
@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("mp,n,eps", [("lambda", 640, 1e-4), ("bbox", 641, 1e-4), ("linear", 767, 0.0),
-                                      ("lambda", 769, 1e-4), ("bbox", 1025, 1e-2), ("lambda", 1664, 1e-4),
+                                      ("lambda", 769, 1e-4), ("bbox", 1025, 1e-2), ("lambda", 1280, 1e-4), ("bbox", 1281, 1e-4),
+                                      ("lambda", 1664, 1e-4),
                                       ("linear", 1793, 1e-4)])
 def test_contraction_edges(gpu, oracle, mp, n, eps):
     """Smallest sizes of both calls, one row past a tile, a super-block and a
@@ -28,7 +29,7 @@ def test_contraction_edges(gpu, oracle, mp, n, eps):
           f"energy {abs(E.item() / e_ref - 1):.2e}")
     assert err.max() <= F_TOL
     assert E.item() == pytest.approx(e_ref, rel=E_TOL)
-    if n >= 1664:   # below, the energy alone keeps the FP32 loop
+    if n >= 1280:   # below, the energy alone keeps the FP32 loop
         assert gpu.atm_energy_raw(to_gpu(x), 1.5, eps, mp).item() == pytest.approx(e_ref, rel=E_TOL)
     gpu.simplex_device_errors()
 
