@@ -275,7 +275,7 @@ int simplex_atm_forces(int64_t n, int64_t d, const float *x, float nu, float eps
  * D_ij = |x_i - x_j|^2 and delta_ij = |y_i - y_j|^2 recomputed from y.
  * x, y: device, n*d FP32.  d_out: device, n(n+1)/2 FP32, or NULL to skip
  * storing D.  loss: device, 1 double (written).
- * prec FP32: from about n^2 (d + 20) = 2e8 (gradient) or 3.6e8 (loss), d <= 96
+ * prec FP32: from about n^2 (d + 20) = 1.5e8 (gradient) or 3.6e8 (loss), d <= 96
  * and no d_out, the pair products run on the tensor cores from FP16 hi + lo
  * splits on a fixed grid (22 bits and more) with FP32 sums, where the workspace
  * has simplex_workspace_bytes(); with less (8 bytes per grid block and 1024 for

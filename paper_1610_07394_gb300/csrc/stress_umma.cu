@@ -445,37 +445,53 @@ __device__ __forceinline__ void load_xt(const CUtensorMap *mh, const CUtensorMap
 // scale4 S_p x_p (k_stress_sx), so no coordinate is loaded here.  This
 // thread: its lane quarter's row, its half of the d coordinates (the sum
 // once, by half 0).  All lanes execute the TMEM loads.
-// F16: dp columns in the accumulator (d of them coordinates, any row
-// alignment), in units of 1/gs (coordinates) and 1/ss (sums).
-template <bool F16>
 __device__ __forceinline__ void flush_g(uint32_t tmem, uint32_t gcol, int B, int quarter, int half,
-                                        int lane, int d, int dp, int64_t n, float scale4, float gs, float ss,
-                                        float *__restrict__ grad, float *__restrict__ S) {
+                                        int lane, int d, int64_t n, float scale4, float *__restrict__ grad,
+                                        float *__restrict__ S) {
+    const uint32_t tl = tmem + ((uint32_t)(32 * quarter) << 16) + gcol;
+    const float s = tmem_ld1(tl + (uint32_t)d);
+    const int64_t row = (int64_t)B * TM + 32 * quarter + lane;
+    const int hw = d >> 1;
+    for (int c = 0; c < hw; c += 16) {
+        float v[16];
+        tmem_ld16(tl + (uint32_t)(half * hw + c), v);
+        if (row < n) {
+            float *gr = grad + row * d + half * hw + c;
+#pragma unroll
+            for (int q = 0; q < 16; q += 4)
+                atomicAdd(reinterpret_cast<float4 *>(gr + q),
+                          make_float4(-scale4 * v[q], -scale4 * v[q + 1], -scale4 * v[q + 2], -scale4 * v[q + 3]));
+        }
+    }
+    if (half == 0 && row < n) atomicAdd(S + row, s);
+}
+
+// The same for F16: dp columns in the accumulator, d of them coordinates (any
+// row alignment), in units of 1/gs (coordinates) and 1/ss (sums).  The
+// truncating sums come out 5e-8 (d >= 16) to 8e-8 (d = 2 to 5) small, measured
+// against 64 bits; the share kShare, under an ulp, moves three quarters of the
+// sums up by one and so gives the mean back.
+__device__ __forceinline__ void flush_g16(uint32_t tmem, uint32_t gcol, int B, int quarter, int half,
+                                          int lane, int d, int dp, int64_t n, float scale4, float gs, float ss,
+                                          float *__restrict__ grad, float *__restrict__ S) {
+    constexpr float kShare = 5.0e-8f;
     const uint32_t tl = tmem + ((uint32_t)(32 * quarter) << 16) + gcol;
     const float s = tmem_ld1(tl + (uint32_t)dp);
     const int64_t row = (int64_t)B * TM + 32 * quarter + lane;
     const int hw = dp >> 1;
-    // F16: the truncating sums come out 2e-8 (d >= 16) to 6e-8 (d = 2) small,
-    // measured against 64 bits; this share of each gives the mean back
-    constexpr float kShare = 3.5e-8f;
-    const float f = F16 ? -scale4 * gs : -scale4, fs = f * kShare;
+    const float f = -scale4 * gs, fs = f * kShare;
     for (int c = 0; c < hw; c += 16) {
         float v[16];
         tmem_ld16(tl + (uint32_t)(half * hw + c), v);
         const int c0 = half * hw + c;
         if (row < n) {
-            if (F16)
 #pragma unroll
-                for (int q = 0; q < 16; ++q) v[q] = fmaf(v[q], f, v[q] * fs);
-            else
-#pragma unroll
-                for (int q = 0; q < 16; ++q) v[q] *= f;
+            for (int q = 0; q < 16; ++q) v[q] = fmaf(v[q], f, v[q] * fs);
             float *gr = grad + row * d + c0;
-            if (!F16 || ((d & 3) == 0 && c0 + 16 <= d)) {
+            if ((d & 3) == 0 && c0 + 16 <= d) {
 #pragma unroll
                 for (int q = 0; q < 16; q += 4)
-                    atomicAdd(reinterpret_cast<float4 *>(gr + q),
-                              make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]));
+                    atomicAdd(reinterpret_cast<float4 *>(gr + q), make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]));
             } else {
 #pragma unroll
                 for (int q = 0; q < 16; ++q)
@@ -483,7 +499,7 @@ __device__ __forceinline__ void flush_g(uint32_t tmem, uint32_t gcol, int B, int
             }
         }
     }
-    if (half == 0 && row < n) atomicAdd(S + row, F16 ? fmaf(s, ss, s * (ss * kShare)) : s);
+    if (half == 0 && row < n) atomicAdd(S + row, fmaf(s, ss, s * (ss * kShare)));
 }
 
 // The same from the centre, one element at a time (any d, any alignment of x).
@@ -856,12 +872,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (t >= 1) {
                 // the previous tile's sides: its columns always, its rows at the end of a run
                 const uint32_t pb = (t - 1) % (uint32_t)ngx;
-                flush_g<F16>(tmem, kGY + NG * (1 + pb), pX, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+                if (F16) flush_g16(tmem, kGY + NG * (1 + pb), pX, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+                else flush_g(tmem, kGY + NG * (1 + pb), pX, quarter, half, lane, d, n, scale4, grad, S);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctl.gxfree[pb]));
                 if (F16 || Y != pY) {
-                    flush_g<F16>(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+                    if (F16) flush_g16(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+                    else flush_g(tmem, kGY, pY, quarter, half, lane, d, n, scale4, grad, S);
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&ctl.gyfree));
@@ -876,9 +894,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!*fail && t >= 1 &&
             mbar_wait(smem_u32(&ctl.g2done), (t - 1) & 1, fail, &g_error)) {
             tc_fence_after();
-            flush_g<F16>(tmem, kGY + NG * (1 + (t - 1) % (uint32_t)ngx), pX, quarter, half, lane, dg, d, n, scale4, gs,
-                         ss, grad, S);
-            flush_g<F16>(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+            const uint32_t gx0 = kGY + NG * (1 + (t - 1) % (uint32_t)ngx);
+            if (F16) {
+                flush_g16(tmem, gx0, pX, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+                flush_g16(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+            } else {
+                flush_g(tmem, gx0, pX, quarter, half, lane, d, n, scale4, grad, S);
+                flush_g(tmem, kGY, pY, quarter, half, lane, d, n, scale4, grad, S);
+            }
         }
     }
     tc_fence_before();
@@ -1420,18 +1443,18 @@ int64_t stress_umma_workspace_bytes(int64_t n, int64_t d, bool bwd) {
 
 static int64_t padded(int64_t d) { return (d + 31) / 32 * 32; }
 
-// Both paths measured: the launches before the main kernel (centre, maxima,
-// operands; the backward's tile scan) cost the F16 path 37 us forward and 58 us
+// Both paths measured: the launches around the main kernel (centre, maxima,
+// operands; the backward's tile scan) cost the F16 path 36 us forward and 40 us
 // backward at any size, the FP32 kernels grow with n^2 (d + 20):
-//   forward   n = 2561, d = 64: 41 against 53 us; 4096, 5: 36 and 42;
+//   forward   n = 2561, d = 64: 40 against 53 us; 4096, 5: 34 and 42;
 //             2560, 20: 38 and 30; 3000, 3: 39 and 29
-//   backward  n = 2560, d = 20: 60 against 66 us; 3000, 3: 54 and 76;
-//             2048, 33: 60 and 57; 2560, 2: 58 and 59
-// n = 10000, d = 64: 78 against 575 us forward, 175 against 1125 us backward;
-// n = 20000, d = 96: 0.26 against 3.35 ms, 0.66 against 7.80 ms.
+//   backward  n = 2048, d = 64: 42 against 64 us; 3000, 3: 41 and 76;
+//             2560, 20: 44 and 66; 1500, 64: 40 and 50
+// n = 10000, d = 64: 79 against 575 us forward, 163 against 1125 us backward;
+// n = 20000, d = 96: 0.26 against 3.35 ms, 0.65 against 7.80 ms.
 bool stress_f16_ok(int64_t n, int64_t d, bool bwd) {
     if (d > summa::kMaxDim || n < 1024) return false;
-    return (double)n * (double)n * (double)(d + 20) >= (bwd ? 2.0e8 : 3.6e8);
+    return (double)n * (double)n * (double)(d + 20) >= (bwd ? 1.5e8 : 3.6e8);
 }
 
 int64_t stress_f16_workspace_bytes(int64_t n, int64_t d, bool bwd) {

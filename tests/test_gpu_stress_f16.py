@@ -29,7 +29,7 @@ def check(gpu, x, y, mp, xt=None):
     assert row_err(gb.double().cpu().numpy(), 2.5 * G).max() <= G_TOL
 
 
-@pytest.mark.parametrize("mp,n,d", [("lambda", 2049, 96), ("bbox", 3072, 95), ("linear", 4097, 1), ("rb", 4224, 3),
+@pytest.mark.parametrize("mp,n,d", [("lambda", 1345, 64), ("lambda", 2049, 96), ("bbox", 3072, 95), ("linear", 4097, 1), ("rb", 4224, 3),
                                     ("lambda", 3000, 31), ("lambda", 2816, 64), ("linear", 3001, 33),
                                     ("lambda", 2600, 97)])
 def test_f16_edges(gpu, mp, n, d):
