@@ -63,6 +63,11 @@ FLOPS_PER_TRIPLE = 20
 # (1), S = Y - X - Z (2), the three derivatives (15) and their sums into the
 # (i,j), (i,k) and (j,k) accumulators (2.5): 53.5.
 FORCE_FLOPS_PER_TRIPLE = 53.5
+# The contraction on the tensor cores (energy from 1280 points, forces from 640):
+# 25 plane products (FMAs) per triple and contracted side, three FP16 hi/lo
+# products each: 150 flops for the energy (one side), 450 for the forces (three).
+CONTRACT_FLOPS_PER_TRIPLE = 150
+CONTRACT_FORCE_FLOPS_PER_TRIPLE = 450
 FP32_LANES_PER_SM = 128
 L2_FLUSH_BYTES = 512 << 20
 PROFILES = os.path.join(ROOT, "profiles")
@@ -506,10 +511,10 @@ def row_edm_n16384_d256(torch, sx, peaks):
     return _edm_big(torch, sx, peaks, x, "bf16x3")
 
 
-def _atm_row(torch, sx, x, maps=("lambda", "bbox", "linear"), steps=3, warmup=1):
-    """ATM energy (pair tables + energy kernel + FP64 reduction) and energy
-    with forces (force tables + forces kernel) per map: whole-call rates,
-    L2 not flushed (the tables of a call are larger than L2 from n = 4096)."""
+def _atm_row(torch, sx, peaks, x, maps=("lambda", "bbox", "linear"), steps=3, warmup=1):
+    """ATM energy (near pairs + operand tiles + contraction, in passes, + FP64
+    reduction) and energy with forces per map: whole-call rates, L2 not flushed
+    (the operands of a call are larger than L2 from n = 4096)."""
     n = len(x)
     r = {"unit": "triplets/s", "triples": triples(n), "n": n}
     e = torch.empty((), dtype=torch.float64, device="cuda")
@@ -529,8 +534,11 @@ def _atm_row(torch, sx, x, maps=("lambda", "bbox", "linear"), steps=3, warmup=1)
         r[k + "_lambda_vs_bbox"] = r[k + "_lambda"] / r[k + "_bbox"]
         if "linear" in maps:
             r[k + "_lambda_vs_linear"] = r[k + "_lambda"] / r[k + "_linear"]
-    r["energy_fp32_frac"] = FLOPS_PER_TRIPLE * r["energy_lambda"] / 1e12 / _fp32_peak(torch)
-    r["energy_forces_fp32_frac"] = FORCE_FLOPS_PER_TRIPLE * r["energy_forces_lambda"] / 1e12 / _fp32_peak(torch)
+    # the FP16 products issued, against the measured BF16 rate (the same pipe)
+    r["energy_tensor_tflops"] = CONTRACT_FLOPS_PER_TRIPLE * r["energy_lambda"] / 1e12
+    r["energy_forces_tensor_tflops"] = CONTRACT_FORCE_FLOPS_PER_TRIPLE * r["energy_forces_lambda"] / 1e12
+    r["energy_tensor_frac"] = r["energy_tensor_tflops"] / peaks["bf16_tflops"]
+    r["energy_forces_tensor_frac"] = r["energy_forces_tensor_tflops"] / peaks["bf16_tflops"]
     return r
 
 
@@ -543,7 +551,7 @@ def _atm_cpu(xh, target):
 def row_atm_n4096(torch, sx, peaks):
     """ATM n=4096 (differentiation config): energy, energy+forces."""
     xh = synth.make_points("atm_n4096")
-    r = _atm_row(torch, sx, torch.from_numpy(xh).cuda())
+    r = _atm_row(torch, sx, peaks, torch.from_numpy(xh).cuda())
     r["cpu_baseline"] = _atm_cpu(xh, 8_000_000)
     return r
 
@@ -553,7 +561,7 @@ def row_atm_n3000(torch, sx, peaks):
     filters, Sec. III-A "approach n from above"), uniform in a cube of side
     20, seed 7."""
     xh = synth.uniform_cube(3000, 3, 20.0, seed=7)
-    r = _atm_row(torch, sx, torch.from_numpy(xh).cuda())
+    r = _atm_row(torch, sx, peaks, torch.from_numpy(xh).cuda())
     r["grid_blocks"] = {mp: sx.simplex_grid_blocks(3, -(-3000 // 32), mp) for mp in ("lambda", "bbox", "linear")}
     r["cpu_baseline"] = _atm_cpu(xh, 4_000_000)
     return r
@@ -563,7 +571,7 @@ def row_atm_n12000(torch, sx, peaks):
     """ATM n=12000 (375 blocks, padded to 512 by lambda), uniform in a cube
     of side 20, seed 8: 2.88e11 triples."""
     xh = synth.uniform_cube(12000, 3, 20.0, seed=8)
-    r = _atm_row(torch, sx, torch.from_numpy(xh).cuda(), steps=2)
+    r = _atm_row(torch, sx, peaks, torch.from_numpy(xh).cuda(), steps=2)
     r["grid_blocks"] = {mp: sx.simplex_grid_blocks(3, -(-12000 // 32), mp) for mp in ("lambda", "bbox", "linear")}
     r["cpu_baseline"] = _atm_cpu(xh, 20_000_000)
     return r
@@ -629,16 +637,14 @@ def row_stress_n65536_d64(torch, sx, peaks):
     ms = _median_ms(torch, lambda: sx.simplex_stress_fwd(x, y, None, loss, "lambda", "fp32", ws), 2)
     r["fwd_lambda"] = pairs / (ms / 1e3)
     g = torch.empty_like(x)
-    ms = _median_ms(torch, lambda: sx.simplex_stress_bwd(x, y, 1.0, g, "lambda", "fp32"), 2)
+    wsb = sx.workspace("stress_bwd", n, w["d"], "lambda")
+    ms = _median_ms(torch, lambda: sx.simplex_stress_bwd(x, y, 1.0, g, "lambda", "fp32", wsb), 2)
     r["bwd_lambda"] = pairs / (ms / 1e3)
-    # algorithmic FP32 flops per pair: forward 4d (two FMAs per coordinate),
+    # algorithmic flops per pair: forward 4d (two FMAs per coordinate),
     # backward 8d (the residual plus the two tile products)
     d = w["d"]
-    fp32 = _fp32_peak(torch)
     r["fwd_tflops"] = 4 * d * r["fwd_lambda"] / 1e12
     r["bwd_tflops"] = 8 * d * r["bwd_lambda"] / 1e12
-    r["fwd_fp32_frac"] = r["fwd_tflops"] / fp32
-    r["bwd_fp32_frac"] = r["bwd_tflops"] / fp32
     r.update(_stress_tensor(torch, sx, peaks, x, y, ("lambda", "bbox", "linear", "rb")))
     w_ = host_cores()
     r["cpu_baseline"] = cpu_stress(xn, yn, list(range(n - 4 * w_, n)), w_)
@@ -812,10 +818,12 @@ def config_block():
     return {"workload": f"ATM triple-dipole energy and adjoint forces (E, F = -dE/dx) over i<j<k, "
                         f"n={w['n']} uniform in a cube of side {w['side']:g}, seed {w['seed']}, nu=1, "
                         f"eps=1e-4 ({triples(w['n'])} triples)",
-            "map": "lambda (two-branch recursive 3-simplex map + J=K plane)",
+            "map": "lambda (2-simplex map of the pair super-blocks; the third index is contracted)",
+            "arithmetic": "FP16 hi + lo products of FP32 pair terms on tensor cores, FP32 sums, FP64 totals; "
+                          "near pairs' triples in FP32",
             "n": w["n"], "triples": triples(w["n"]),
             "l2": f"flushed before every timed step ({L2_FLUSH_BYTES >> 20} MB write); the call's "
-                  f"force tables (9.7 GB) exceed L2 as well"}
+                  f"operand tiles (7.5 GB) exceed L2 as well"}
 
 
 def headline_cpu_rows(n, workers):
@@ -907,8 +915,8 @@ def our_arm(args):
     torch.cuda.synchronize()
     # the timed steps run without the library's event pairs (profile(1) then
     # (0) clears the counters; the launch counter keeps counting), and a
-    # second pass of a few steps with the event pairs on times the forces
-    # kernel for the roofline
+    # second pass of a few steps with the event pairs on times the
+    # contraction kernel for the roofline
     sx.simplex_profile(True)
     sx.simplex_profile(False)
     times = time_steps(torch, step, args.steps, 0, flush, label="energy_forces_lambda")
@@ -922,7 +930,8 @@ def our_arm(args):
         dist.barrier()
     value, ms_step = job_rate(sum(times) / len(times), units, world, dist, "cuda")
     k_ms = main_ms / max(main_k, 1)
-    achieved = FORCE_FLOPS_PER_TRIPLE * units / (k_ms / 1e3) / 1e12
+    achieved = CONTRACT_FORCE_FLOPS_PER_TRIPLE * units / (k_ms / 1e3) / 1e12
+    tensor_peak = peaks["bf16_tflops"]
     e_step = float(e.item())
     f_step = f.cpu().numpy()
 
@@ -969,21 +978,26 @@ def our_arm(args):
     rows = rows_measure(torch, sx, peaks) if (do_rows and rank == 0) else None
     clk = clocks.stop()
 
-    traffic, traffic_note = stated_traffic("k_atm_forces_n16384.md")
+    traffic, traffic_note = stated_traffic("k_atm_umma.md")
     line = {
         "metric": METRIC, "value": value, "unit": "triplets/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_step,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
         "data": "synthetic", "config": config_block(),
         "maps": maps,
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
-                     "frac": achieved / fp32_peak, "traffic": traffic, "traffic_source": traffic_note,
+        "roofline": {"bound": "tensor", "achieved": achieved, "peak": tensor_peak, "unit": "TFLOP/s",
+                     "frac": achieved / tensor_peak,
+                     "frac_of_sustained": achieved / peaks.get("bf16_tflops_sustained", tensor_peak),
+                     "traffic": traffic, "traffic_source": traffic_note,
                      "algorithmic_bytes": 12 * n + 24 * n + 8,
-                     "kernel": "k_atm_forces<lambda>", "kernel_ms": k_ms,
-                     "flops_per_triple": FORCE_FLOPS_PER_TRIPLE,
-                     "peak_basis": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {sm_max:g} MHz "
-                                   f"(unit counts and max clock; the {peak_src} peaks file has no FP32 "
-                                   f"figure)"},
+                     "kernel": "k_atm_umma<forces>", "kernel_ms": k_ms,
+                     "flops_per_triple": CONTRACT_FORCE_FLOPS_PER_TRIPLE,
+                     "fp32_equivalent_tflops": FORCE_FLOPS_PER_TRIPLE * units / (k_ms / 1e3) / 1e12,
+                     "fp32_peak": fp32_peak,
+                     "peak_basis": f"cuBLAS BF16 rate of the {peak_src} peaks file (FP16 products run on the "
+                                   f"same pipe); fp32_equivalent_tflops counts the FP32 triple loop's "
+                                   f"{FORCE_FLOPS_PER_TRIPLE} flops per triple, fp32_peak is {sms} SMs x "
+                                   f"{FP32_LANES_PER_SM} lanes x 2 x {sm_max:g} MHz"},
         "e2e": e2e,
         "gpu_launches": launches,
         "clocks": clk,

@@ -17,8 +17,9 @@
 // two triples on the FMA pipe, which bounds it at 65-70% of its issue rate
 // with the tensor cores idle.  Energy and forces, before and after:
 // n = 1024 297 -> 152 us, n = 3000 6.47 -> 1.56 ms, n = 4096 15.4 -> 3.77 ms,
-// n = 16384 960 -> 240 ms (1390 TFLOP/s of FP16 products, the tensor pipe 85%
-// busy at the 1.64 GHz that the power limit leaves); energy alone
+// n = 16384 960 -> 210 ms (1570 TFLOP/s of FP16 products, 93% of the sustained
+// cuBLAS BF16 rate; at n = 4096 the tensor pipe is 86% busy at the 1.63 GHz that
+// the power limit leaves); energy alone
 // n = 3000 2.18 -> 0.85 ms, n = 4096 5.16 -> 1.69 ms.
 //
 // Near pairs.  Each point's pair with its nearest neighbour is left out of the
@@ -183,9 +184,10 @@ struct Walk {
     const Work &W;
     const int *list;
     int c, C, phase, nl;
+    bool full;        // every cluster has a segment in this row of the deal
     int64_t t, nL, nS;
     __device__ Walk(const Work &w, const int *l)
-        : W(w), list(l), c((int)(blockIdx.x >> 1)), C((int)(gridDim.x >> 1)), phase(0), t(0) {
+        : W(w), list(l), c((int)(blockIdx.x >> 1)), C((int)(gridDim.x >> 1)), phase(0), full(false), t(0) {
         nl = 3 * (6 / w.G);
         nL = (int64_t)nl * w.S;
         nS = (int64_t)7 * w.S;
@@ -203,11 +205,13 @@ struct Walk {
         const int rem = (int)(nL % C);
         if (phase == 0) {
             idx = c + C * t;
+            full = C * (t + 1) <= nL;
             if (idx < nL) { ++t; return true; }
             phase = rem && c >= rem ? 1 : 2;
             t = 0;
         }
         const int64_t head = rem ? (int64_t)(C - rem) * W.G : 0;
+        full = false;
         if (phase == 1) {
             idx = t * (C - rem) + (c - rem);
             if (t < W.G && idx < nS) { ++t; idx += nL; return true; }
@@ -216,6 +220,7 @@ struct Walk {
         }
         idx = head + c + C * t;
         if (idx >= nS) return false;
+        full = head + C * (t + 1) <= nS;
         ++t;
         idx += nL;
         return true;
@@ -269,10 +274,13 @@ __global__ void __launch_bounds__(256) k_atm_prep(int64_t n, const float *__rest
                                                   int gx, int cells, bool rows, float *__restrict__ uinv,
                                                   int *__restrict__ nn,
                                                   int *__restrict__ list, double *__restrict__ near_energy,
-                                                  double *__restrict__ forces) {
+                                                  unsigned long long *__restrict__ pace, double *__restrict__ forces) {
     const int lane = threadIdx.x & 31;
     const int64_t gt = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (gt == 0) *near_energy = 0.0;
+    if (gt == 0) {
+        *near_energy = 0.0;
+        *pace = 0ull;
+    }
     if (gt < cells) {
         const int wy = (int)(gt / gx), wx = (int)(gt - (int64_t)wy * gx);
         const List2 L = decode2<MAP>((uint32_t)wx, (uint32_t)wy, ns);
@@ -639,6 +647,28 @@ __global__ void __launch_bounds__(256) k_atm_tiles(int64_t n, const float *__res
 
 // ---------------------------------------------------------------- contraction
 
+// The clusters keep pace where the operands exceed the L2 cache: every kPace
+// chunks a cluster that is ahead waits for the others, so that the chunk's
+// tiles, which neighbouring super-blocks share, are read from HBM once and not
+// once per cluster (they drift apart by more than the cache holds: n = 16384
+// read 1.28 TB, 73% of what the SMs ask for, against 0.25 TB with the pace
+// kept, and took 239 ms against 210).  A matter of speed only, nothing else
+// depends on the count: the wait ends after kPaceCycles (0.5 ms) whether the
+// others have come or not, and a cluster whose wait ran out (some others are
+// not running) keeps no pace from there on.
+constexpr int kPace = 64;
+constexpr long long kPaceCycles = 1000000;
+
+__device__ __forceinline__ bool keep_pace(unsigned long long *ctr, unsigned long long target) {
+    atomicAdd(ctr, 1ull);
+    const long long t0 = clock64();
+    while (*reinterpret_cast<volatile unsigned long long *>(ctr) < target) {
+        if (clock64() - t0 > kPaceCycles) return false;
+        __nanosleep(100);
+    }
+    return true;
+}
+
 struct Ctl {
     uint64_t full[NS], empty[NS];   // ring: copies -> MMA -> copies
     uint64_t pfull[NS];             // first CTA: the peer's copies of a stage have landed
@@ -718,7 +748,7 @@ template <bool FORCES>
 __global__ void __launch_bounds__(kThreads, 1)
     k_atm_umma(const __grid_constant__ CUtensorMap mT, int64_t n, const float *__restrict__ x, float nu, float eps,
                Work W, const int *__restrict__ list, const float *__restrict__ uinv, const int *__restrict__ nn,
-               double *__restrict__ partials, double *__restrict__ forces) {
+               unsigned long long *__restrict__ pace, double *__restrict__ partials, double *__restrict__ forces) {
     constexpr bool UPPER = !FORCES;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
@@ -757,6 +787,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             Walk<UPPER> walk(W, list);
             uint32_t it = 0;
+            unsigned long long paced = 0;
             Seg g;
             bool ok = true;
             while (ok && !*fail && walk.next(g)) {
@@ -765,6 +796,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                     int pa, pb;
                     planes_of(g.o, g.t0 + t, pa, pb);
                     for (int c = g.c0; c < g.c1; ++c) {
+                        if (FORCES && pace && rank == 0 && walk.full && c % kPace == 0 &&
+                            !keep_pace(pace, paced += (unsigned long long)walk.C))
+                            pace = nullptr;
                         const uint32_t s = it % NS, ph = (it / NS) & 1;
                         // free once the pair's MMAs have read the stage
                         if (!(ok = mbar_wait(smem_u32(&ctl.empty[s]), ph ^ 1, fail, &g_error))) break;
@@ -1031,7 +1065,7 @@ static int smem_optin(int &clusters) {
 template <bool FORCES>
 static cudaError_t launch(int clusters, cudaStream_t s, const CUtensorMap &mT, int64_t n, const float *x, float nu,
                           float eps, const Work &W, const int *list, const float *uinv, const int *nn,
-                          double *partials, double *forces) {
+                          unsigned long long *pace, double *partials, double *forces) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * clusters));
     cfg.blockDim = dim3(kThreads);
@@ -1044,13 +1078,13 @@ static cudaError_t launch(int clusters, cudaStream_t s, const CUtensorMap &mT, i
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_atm_umma<FORCES>, mT, n, x, nu, eps, W, list, uinv, nn, partials, forces);
+    return cudaLaunchKernelEx(&cfg, k_atm_umma<FORCES>, mT, n, x, nu, eps, W, list, uinv, nn, pace, partials, forces);
 }
 
 // Room behind the tables: the list of super-blocks, the row scales and the
 // FP64 partials (one per CTA and pass) with the reduction's slots.
 struct Rest {
-    int64_t list, uinv, nn, part, total;
+    int64_t list, uinv, nn, pace, part, total;
 };
 constexpr int kMaxCtas = 256;
 
@@ -1060,7 +1094,8 @@ static Rest rest_of(int64_t n, int passes) {
     r.list = 0;
     r.uinv = align_up(4 * (ns * (ns + 1) / 2), 256);
     r.nn = r.uinv + align_up(4 * n, 256);
-    r.part = r.nn + align_up(4 * n, 256);   // [near pairs' energy][per CTA and pass]
+    r.pace = r.nn + align_up(4 * n, 256);
+    r.part = r.pace + 16;   // [near pairs' energy][per CTA and pass]
     r.total = r.part + 8 * (1 + (int64_t)kMaxCtas * passes + kReduceSlots);
     return r;
 }
@@ -1123,6 +1158,10 @@ int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float ep
     float *uinv = (float *)(rb + R.uinv);
     int *nn = (int *)(rb + R.nn);
     double *near_energy = (double *)(rb + R.part), *partials = near_energy + 1;
+    // operands (28 bytes per ordered pair) well beyond the 126 MB of L2 (n = 3000,
+    // 252 MB: 1.56 ms without, 1.59 with; 4096: 3.77 both ways; 16384 above)
+    unsigned long long *pace_ctr = (unsigned long long *)(rb + R.pace);
+    unsigned long long *pace = want_forces && n > 4096 ? pace_ctr : nullptr;
     const Grid g2 = grid2(ns, map);
     const int cells = (int)(g2.gx * g2.gy);
     int st, clusters = 0;
@@ -1130,9 +1169,9 @@ int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float ep
     const unsigned pb = (unsigned)((n + 7) / 8);
     double *fz = want_forces ? forces : nullptr;
     const bool rows = !want_forces && ns <= 24;
-    if (map == MAP_LAMBDA) k_atm_prep<MAP_LAMBDA><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, fz);
-    else if (map == MAP_BBOX) k_atm_prep<MAP_BBOX><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, fz);
-    else k_atm_prep<MAP_LINEAR><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, fz);
+    if (map == MAP_LAMBDA) k_atm_prep<MAP_LAMBDA><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, pace_ctr, fz);
+    else if (map == MAP_BBOX) k_atm_prep<MAP_BBOX><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, pace_ctr, fz);
+    else k_atm_prep<MAP_LINEAR><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, pace_ctr, fz);
     // near pairs: 128 pairs by `seg` points per block, enough blocks for the chip
     const int seg = n < 2048 ? 16 : n < 4096 ? 32 : 128;
     const dim3 ng((unsigned)((n + kNearThreads - 1) / kNearThreads), (unsigned)((n + seg - 1) / seg));
@@ -1160,8 +1199,8 @@ int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float ep
         if (!make_map_rows16(&mT, tab, tile_sets(W.T) * PLANES * 2 * TM, 2 * TM)) return SIMPLEX_ECUDA;
         prof_begin(s);
         const cudaError_t e =
-            want_forces ? launch<true>(clusters, s, mT, n, x, nu, eps, W, list, uinv, nn, energy ? partials : nullptr, forces)
-                        : launch<false>(clusters, s, mT, n, x, nu, eps, W, list, uinv, nn, partials + (int64_t)p * 2 * clusters, nullptr);
+            want_forces ? launch<true>(clusters, s, mT, n, x, nu, eps, W, list, uinv, nn, pace, energy ? partials : nullptr, forces)
+                        : launch<false>(clusters, s, mT, n, x, nu, eps, W, list, uinv, nn, nullptr, partials + (int64_t)p * 2 * clusters, nullptr);
         prof_end(s);
         note_launches(1);
         if (e != cudaSuccess) return cuda_status(e);
