@@ -4,14 +4,14 @@
 Headline workload (one "step"): the Axilrod-Teller-Muto triple-dipole energy
 and its adjoint forces F = -dE/dx over all i < j < k of n = 16384 points
 uniform in a cube of side 20 (seed 6), nu = 1, eps = 1e-4: 732,873,539,584
-triples on the lambda-mapped 3-simplex grid (two-branch recursive map plus
-the J = K plane), one call of simplex_atm_forces (force tables over the
-2-simplex of blocks, the forces kernel, the FP64 reduction of the energy),
-FP32 per triple, FP64 force and energy sums.  Metric: triples per second
-(whole job), with the same step timed for the bounding-box and linear
-(cube-root) maps, the forces kernel timed live against the FP32 ALU
-roofline, an end-to-end number through the C ABI with host buffers, and the
-FP64 CPU oracle timed on all host cores (a bounded sample, extrapolated).
+triples, one call of simplex_atm_forces (the near pairs' triples in FP32, the
+operand tiles, the contraction over the super-blocks of pairs that the
+2-simplex map lists, the FP64 reduction of the energy), FP32 terms, FP64
+force and energy sums.  Metric: triples per second (whole job), with the same
+step timed for the bounding-box and linear maps, the contraction kernel timed
+live against the tensor-core rate, an end-to-end number through the C ABI
+with host buffers, and the FP64 CPU oracle timed on all host cores (a bounded
+sample, extrapolated).
 
 ``--rows`` (default on at one GPU) also times every other kernel on the path
 at its own configuration (coverage m = 2, 3, 4; EDM n = 1024 d = 3,
