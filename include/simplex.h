@@ -72,9 +72,9 @@ typedef enum {
 } simplex_map;
 
 typedef enum {
-    SIMPLEX_PREC_FP32 = 0,    /* FP32 accuracy: every step in FP32, or for the
-                                 stress at size FP16 hi + lo products that err
-                                 no more (simplex_stress_fwd)                */
+    SIMPLEX_PREC_FP32 = 0,    /* every step in FP32, or for the stress at size
+                                 FP16 hi + lo products with FP32 sums
+                                 (simplex_stress_fwd)                        */
     SIMPLEX_PREC_BF16X3 = 1,  /* Gram term on tensor cores, split BF16 hi+lo */
     SIMPLEX_PREC_AUTO = 2     /* library choice by d                          */
 } simplex_prec;
@@ -277,9 +277,14 @@ int simplex_atm_forces(int64_t n, int64_t d, const float *x, float nu, float eps
  * storing D.  loss: device, 1 double (written).
  * prec FP32: from about n^2 (d + 20) = 1.5e8 (gradient) or 3.6e8 (loss), d <= 96
  * and no d_out, the pair products run on the tensor cores from FP16 hi + lo
- * splits on a fixed grid (22 bits and more) with FP32 sums, where the workspace
- * has simplex_workspace_bytes(); with less (8 bytes per grid block and 1024 for
- * a loss, none for the gradient alone) every step stays in FP32.
+ * splits with FP32 sums, where the workspace has simplex_workspace_bytes(); with
+ * less (8 bytes per grid block and 1024 for a loss, none for the gradient alone)
+ * every step stays in FP32, the caller's choice.  The splits keep 22 bits of a
+ * point's largest entry after every coordinate is scaled to one size: errors
+ * as in FP32 where coordinates or points differ in size (shared wide axes,
+ * groups far apart, single far points, to 10^4 and within twice FP32's), up to
+ * ten times FP32's in single columns of the gradient where the entries of a
+ * point do so on their own (heavy-tailed in every entry).
  */
 int simplex_stress_fwd(int64_t n, int64_t d, const float *x, const float *y,
                        float *d_out, double *loss, int map, int prec,

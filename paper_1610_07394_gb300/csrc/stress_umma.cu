@@ -82,13 +82,15 @@ struct Ctl {
     uint32_t tmem;
     int fail;
     alignas(16) float acol[kEpiWarps][64];    // a_j of each epilogue warp's 64 columns
+    alignas(16) float wcol[kEpiWarps][64];    // FP16: their w_j
+    alignas(16) float ix[96];                 // FP16: inverse scales of the coordinates
     float red[2 * (kThreads / 32)];
 };
 
-constexpr int kCtlBytes = 4096;
+constexpr int kCtlBytes = 5120;
 constexpr int SMEM_BYTES = 1024 + kStages * STAGE_BYTES + C_BYTES + kCtlBytes;
 static_assert(sizeof(Ctl) <= kCtlBytes, "control block");
-static_assert(offsetof(Ctl, acol) % 16 == 0, "float4 reads of a_j");
+static_assert(offsetof(Ctl, acol) % 16 == 0 && offsetof(Ctl, wcol) % 16 == 0 && offsetof(Ctl, ix) % 16 == 0, "float4 reads");
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory per block");
 
 // The tiles a CTA handles.  The map's grid (gx x gy, x fastest) lists the
@@ -304,103 +306,218 @@ struct ChunkWalk {
 // ---------------------------------------------------------------- FP32 on the tensor cores
 //
 // SIMPLEX_PREC_FP32 with the products on the tensor cores (F16 = true): the
-// operands are split into FP16 hi + lo on one fixed grid each.  S is scaled by
-// the power of two that takes the largest |S| of all points to [2^10, 2^11),
-// hi = the nearest integer (11 bits, exact in FP16), lo = the rest rounded to
-// 11 bits: 2^-24 of that largest; Delta likewise.  hi.hi is then a sum of
-// integers, exact in the tensor core's truncating FP32 sums up to 2^24, and
-// has an accumulator of its own; the three other products, 2^-11 of it, have
-// another.  So the residuals carry no truncation (in one accumulator all of M
-// came out 1e-7 small, and the loss with it).  The second product's operands
-// (the residual tile C, X) are rounded to FP16 hi + lo of 22 bits, scaled into
-// FP16's range by bounds on |r| and |x|; both sides are flushed for every
-// tile, so that no truncating sum runs over more than 128 points.  The
-// residuals and the gradient do not change when x and y move together, so
-// both are taken from a centre c (the mean of 64 points): the products' size
-// is then the cloud's, wherever it lies.  Against 64 bits, N(0,1) clouds of
-// n = 2560 to 20000, d = 2 to 96: loss 1e-10 to 5e-9 as with the FP32 kernels,
-// gradient 1.0e-7 to 2.0e-7 of its norm (1.0e-7 to 2.9e-7); a cloud 20 times its
-// width away from the origin 1e-7 to 2e-7 (6e-7 to 1.7e-6).
-constexpr int kCentre = 64;   // points of the mean
+// operands are split into FP16 hi + lo on an integer grid of each point.  The
+// point's S and Delta are scaled by powers of two that take its largest entry
+// to [2^10, 2^11), hi = the nearest integer (11 bits, exact in FP16), lo = the
+// rest rounded to 11 bits.  hi.hi is then a sum of integers, exact in the
+// tensor core's truncating FP32 sums up to 2^24, and has an accumulator of its
+// own; the three other products, 2^-11 of it, have another.  So the residuals
+// carry no truncation (in one accumulator all of M came out 1e-7 small, and the
+// loss with it).
+//
+// The scales.  An entry far below its point's largest keeps fewer bits, so the
+// entries of a point are brought to one size first.  Coordinate t: S_t is
+// divided by its largest |S_t| over all points (a power of two, like every scale
+// here) and Delta_t multiplied by it, which leaves the products S_t Delta_t, and
+// so M, as they are: a wide coordinate that x and y share (Delta_t = 0) takes no
+// bits from the narrow ones, and what is left differs between coordinates as
+// their parts of the residual do.  Delta is scaled to the size of S, by the
+// means of 64 points (by the largest, a single large displacement would take
+// the others' bits).  The scale of a point p is kept as w_p, M_ij = odd w_i w_j
+// times the accumulators (odd: a factor that two equal ones cannot give).  With
+// one grid for all points and coordinates, a shared axis 10^3 times wider than
+// the others left 5e-6 in the gradient's norm and 3e-3 in its worst row (FP32
+// kernels 1e-7 and 3e-5; so now).  Entries of a point that differ on their own
+// (every entry heavy-tailed) keep fewer bits: up to ten times the FP32 kernels'
+// error in single columns of the gradient.
+//
+// The second product's operands (the residual tile C, X) are rounded to FP16
+// hi + lo of 22 bits, scaled into FP16's range by bounds on |r| and, per
+// coordinate, on |x|; both sides are flushed for every tile, so that no
+// truncating sum runs over more than 128 points.  The residuals and the
+// gradient do not change when x and y move together, so both are taken from a
+// centre c (the mean of 64 points): the products' size is then the cloud's,
+// wherever it lies.
+constexpr int kCentre = 64;   // points of the means
 constexpr int kMaxDim = 96;
 
+// Written by the passes before the main kernel, d entries each:
+struct Stats {
+    float c[kMaxDim];                                         // centre
+    float ms[kMaxDim], md[kMaxDim];                           // mean |S_t|, |Delta_t| of its points
+    uint32_t xs[kMaxDim], xd[kMaxDim], xx[kMaxDim];           // largest |S_t|, |Delta_t|, |x_t| (bits)
+    float ix[kMaxDim];                                        // inverse scales of x_t (0 beyond d)
+    float cs, ic;                                             // scale of the residuals and its inverse
+    float odd;                                                // 1 or 1/2, see w
+};
+constexpr int64_t kStatsBytes = 4096;
+static_assert(sizeof(Stats) <= kStatsBytes, "statistics block");
+
+__device__ __forceinline__ float pow2(int e) { return ldexpf(1.0f, e > 120 ? 120 : (e < -120 ? -120 : e)); }
+
+// e with m < 2^e, m >= 2^(e-1); `none` for 0, infinity and NaN.
+__device__ __forceinline__ int exponent_of(float m, int none) {
+    int e = none;
+    if (m > 0.f && m <= 3.4e38f) frexpf(m, &e);
+    return e;
+}
+
+// The scales of coordinate t (powers of two) for S, Delta and x, in shared
+// memory, and the exponent of w for a point of scale 1.
 struct Scales {
-    float s, d, x, c;        // of S, Delta, x and the residuals
-    float is, id, ix, ic;    // their inverses
+    float s[kMaxDim], d[kMaxDim], x[kMaxDim];
+    int half;
+    float cs;   // of the residuals
 };
 
-// mx: the bits of the largest |S|, |Delta|, |x|.
-__device__ __forceinline__ float pow2_scale(float m, int top) {
-    int e = 0;
-    if (m > 0.f && m <= 3.4e38f) frexpf(m, &e);   // m < 2^e; 0, inf and NaN take 1
-    e = top - e;
-    return ldexpf(1.0f, e > 100 ? 100 : (e < -100 ? -100 : e));
+__device__ __forceinline__ int warp_max(int v) { return __reduce_max_sync(0xffffffffu, v); }
+__device__ __forceinline__ float warp_maxf(float v) {   // (not negative, not NaN)
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+__device__ __forceinline__ bool finite_bits(float v) { return v <= 3.4e38f; }
+
+// One warp; `out` (if given) gets what the main kernel needs.  A coordinate
+// whose S or Delta is 0 for every point takes no part in M (scales 0).
+__device__ __forceinline__ void find_scales(const Stats *st, int d, int lane, Scales &q, Stats *out) {
+    constexpr int kNone = -100000;
+    constexpr int K = kMaxDim / 32;
+    float xs[K], xd[K], ms[K], md[K], xx[K];
+    int es[K];
+    bool use[K];
+    float big = 0.f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int t = lane + 32 * k;
+        const bool in = t < d;
+        xs[k] = in ? __uint_as_float(st->xs[t]) : 0.f;
+        xd[k] = in ? __uint_as_float(st->xd[t]) : 0.f;
+        xx[k] = in ? __uint_as_float(st->xx[t]) : 0.f;
+        ms[k] = in ? st->ms[t] : 0.f;
+        md[k] = in ? st->md[t] : 0.f;
+        use[k] = xs[k] != 0.f && xd[k] != 0.f;
+        if (use[k] && finite_bits(xs[k])) big = fmaxf(big, xs[k]);
+    }
+    big = warp_maxf(big);
+    // Exponents of the coordinates' sizes, counted from the widest: rounded so
+    // that coordinates of about one size (0.6 to 1 of it) share one scale.
+    const int eb = exponent_of(big, 0);
+    int top = kNone;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        es[k] = eb;
+        if (use[k] && finite_bits(xs[k])) es[k] = eb - 1 + exponent_of(fmaxf(xs[k] / big, 1e-37f) * 1.6818f, 1);
+        if (use[k] && finite_bits(xd[k])) top = max(top, exponent_of(xd[k], kNone) + es[k]);
+    }
+    top = warp_max(top);
+    // sizes of S_t 2^-es and Delta_t 2^(es - top), and
+    // |r| <= 4 sum_t max|S_t| max|Delta_t| < 2^15 / cs
+    float size_s = 0.f, size_d = 0.f, sum = 0.f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if (!use[k] || top == kNone) continue;
+        const int down = max(es[k] - top, -200);
+        if (finite_bits(ms[k])) size_s = fmaxf(size_s, ldexpf(ms[k], -es[k]));
+        if (finite_bits(md[k])) size_d = fmaxf(size_d, ldexpf(md[k], down));
+        if (finite_bits(xs[k]) && finite_bits(xd[k])) sum += ldexpf(xs[k], -es[k]) * ldexpf(xd[k], down);
+    }
+    size_s = warp_maxf(size_s);
+    size_d = warp_maxf(size_d);
+    sum = warp_sum_f32(sum);
+    const float ratio = (size_s > 0.f ? size_s : 1.0f) / fmaxf(size_d > 0.f ? size_d : 1.0f, 1e-30f);
+    const int e = top == kNone ? 0 : exponent_of(ratio * 1.4142136f, 1) - 1 - top;   // of Delta against S
+    const int er = sum > 0.f ? exponent_of(sum, 0) + 2 + top : 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int t = lane + 32 * k;
+        const int ex = exponent_of(xx[k], 0);
+        q.s[t] = use[k] ? pow2(-es[k]) : 0.f;
+        q.d[t] = use[k] ? pow2(es[k] + e) : 0.f;
+        q.x[t] = pow2(11 - ex);
+        if (out) out->ix[t] = t < d ? pow2(ex - 11) : 0.f;
+    }
+    if (lane == 0) {
+        q.half = -(e >> 1);   // 2^-e = 2^half 2^half 2^-odd
+        q.cs = pow2(15 - er);
+        if (out) {
+            out->odd = pow2(-(e & 1));
+            out->cs = pow2(15 - er);
+            out->ic = pow2(er - 15);
+        }
+    }
 }
 
-__device__ __forceinline__ Scales scales_of(const uint32_t *mx, int d) {
-    const float ms = __uint_as_float(__ldg(mx)), md = __uint_as_float(__ldg(mx + 1)), mxx = __uint_as_float(__ldg(mx + 2));
-    Scales q;
-    q.s = pow2_scale(ms, 11);
-    q.d = pow2_scale(md, 11);
-    q.x = pow2_scale(mxx, 11);
-    // |r| <= 4 d max|S| max|Delta| < 2^15 / c
-    int es = 0, ed = 0;
-    if (ms > 0.f && ms <= 3.4e38f) frexpf(ms, &es);
-    if (md > 0.f && md <= 3.4e38f) frexpf(md, &ed);
-    int e = 15 - (es + ed + 2 + (32 - __clz(d)));
-    q.c = ldexpf(1.0f, e > 100 ? 100 : (e < -100 ? -100 : e));
-    q.is = 1.0f / q.s; q.id = 1.0f / q.d; q.ix = 1.0f / q.x; q.ic = 1.0f / q.c;
-    return q;
-}
-
-// c, and zeroed maxima (one block of 8 x 96 threads).
-__global__ void __launch_bounds__(8 * kMaxDim) k_stress_centre(const float *__restrict__ x, int64_t n, int d,
-                                                               float *__restrict__ c, uint32_t *__restrict__ mx) {
-    __shared__ float part[8][kMaxDim];
+// c, the means around it and zeroed maxima (one block of 8 x 96 threads).
+__global__ void __launch_bounds__(8 * kMaxDim) k_stress_centre(const float *__restrict__ x, const float *__restrict__ y,
+                                                               int64_t n, int d, Stats *st) {
+    __shared__ float part[8][kMaxDim], part2[8][kMaxDim];
     const int t = threadIdx.x % kMaxDim, g = threadIdx.x / kMaxDim;
-    float v = 0.f;
-    if (t < d)
-        for (int k = g; k < kCentre; k += 8) v += __ldg(x + (n * k / kCentre) * d + t) * (1.0f / kCentre);
+    float xv[kCentre / 8], yv[kCentre / 8], v = 0.f;
+#pragma unroll
+    for (int k = 0; k < kCentre / 8; ++k) {
+        const int64_t p = n * (g + 8 * k) / kCentre;
+        xv[k] = t < d ? __ldg(x + p * d + t) : 0.f;
+        yv[k] = t < d ? __ldg(y + p * d + t) : 0.f;
+        v += xv[k] * (1.0f / kCentre);
+    }
     part[g][t] = v;
+    __syncthreads();
+    float c = part[0][t];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) c += part[k][t];
+    __syncthreads();
+    float ms = 0.f, md = 0.f;
+#pragma unroll
+    for (int k = 0; k < kCentre / 8; ++k) {
+        ms += fabsf((xv[k] - c) + (yv[k] - c)) * (1.0f / kCentre);
+        md += fabsf(xv[k] - yv[k]) * (1.0f / kCentre);
+    }
+    part[g][t] = ms;
+    part2[g][t] = md;
     __syncthreads();
     if (g == 0) {
 #pragma unroll
-        for (int k = 1; k < 8; ++k) v += part[k][t];
-        c[t] = v;
+        for (int k = 1; k < 8; ++k) {
+            ms += part[k][t];
+            md += part2[k][t];
+        }
+        st->c[t] = c;
+        st->ms[t] = ms;
+        st->md[t] = md;
+        st->xs[t] = st->xd[t] = st->xx[t] = 0u;
     }
-    if (threadIdx.x < 3) mx[threadIdx.x] = 0u;
 }
 
-// Largest |S|, |Delta|, |x - c| (as bits: NaN above infinity above all numbers).
-// Bound by load latency and by the updates of three addresses: each block
-// updates them once, after a maximum in shared memory (once per warp, at two
-// blocks an SM: forward pass of n = 16384, d = 33 in 139.1 us; now 136.0).
+// Largest |S_t|, |Delta_t|, |x_t - c_t| of every coordinate (as bits: NaN above
+// infinity above all numbers).  A thread keeps to one coordinate (the stride is
+// a multiple of d), a block updates each address once, after a maximum in
+// shared memory.  Bound by load latency at these sizes.
 __global__ void __launch_bounds__(256) k_stress_max(const float *__restrict__ x, const float *__restrict__ y,
-                                                    int64_t count, int d, const float *__restrict__ c,
-                                                    uint32_t *__restrict__ mx) {
-    __shared__ uint32_t best[3];
-    uint32_t m[3] = {0u, 0u, 0u};
-    const int64_t e0 = (int64_t)blockIdx.x * 256 + threadIdx.x, step = (int64_t)gridDim.x * 256;
-    int t = (int)(e0 % d);
-    const int dt = (int)(step % d);
-    if (threadIdx.x < 3) best[threadIdx.x] = 0u;
+                                                    int64_t count, int d, Stats *st) {
+    __shared__ uint32_t best[3][kMaxDim];
+    for (int k = threadIdx.x; k < 3 * kMaxDim; k += 256) (&best[0][0])[k] = 0u;
     __syncthreads();
+    const int width = 256 / d * d;   // threads at work: whole rows of coordinates
+    const int t = threadIdx.x % d;
+    if ((int)threadIdx.x < width) {
+        uint32_t m[3] = {0u, 0u, 0u};
+        const float ct = st->c[t];
+        const int64_t step = (int64_t)gridDim.x * width;
 #pragma unroll 4
-    for (int64_t e = e0; e < count; e += step) {
-        const float ct = __ldg(c + t), a = __ldg(x + e), b = __ldg(y + e);
-        m[0] = max(m[0], __float_as_uint(fabsf((a - ct) + (b - ct))));
-        m[1] = max(m[1], __float_as_uint(fabsf(a - b)));
-        m[2] = max(m[2], __float_as_uint(fabsf(a - ct)));
-        t += dt;
-        if (t >= d) t -= d;
-    }
+        for (int64_t e = (int64_t)blockIdx.x * width + threadIdx.x; e < count; e += step) {
+            const float a = __ldg(x + e), b = __ldg(y + e);
+            m[0] = max(m[0], __float_as_uint(fabsf((a - ct) + (b - ct))));
+            m[1] = max(m[1], __float_as_uint(fabsf(a - b)));
+            m[2] = max(m[2], __float_as_uint(fabsf(a - ct)));
+        }
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        m[k] = __reduce_max_sync(0xffffffffu, m[k]);
-        if ((threadIdx.x & 31) == 0) atomicMax(best + k, m[k]);
+        for (int k = 0; k < 3; ++k) atomicMax(&best[k][t], m[k]);
     }
     __syncthreads();
-    if (threadIdx.x < 3 && best[threadIdx.x]) atomicMax(mx + threadIdx.x, best[threadIdx.x]);
+    if ((int)threadIdx.x < d) {
+        if (best[0][threadIdx.x]) atomicMax(st->xs + threadIdx.x, best[0][threadIdx.x]);
+        if (best[1][threadIdx.x]) atomicMax(st->xd + threadIdx.x, best[1][threadIdx.x]);
+        if (best[2][threadIdx.x]) atomicMax(st->xx + threadIdx.x, best[2][threadIdx.x]);
+    }
 }
 
 // hi and lo of a value on the integer grid.
@@ -476,26 +593,31 @@ __device__ __forceinline__ void flush_g(uint32_t tmem, uint32_t gcol, int B, int
 }
 
 // The same for F16: dp columns in the accumulator, d of them coordinates (any
-// row alignment), in units of 1/gs (coordinates) and 1/ss (sums).  The
-// truncating sums come out 5e-8 (d >= 16) to 8e-8 (d = 2 to 5) small, measured
+// row alignment), in units of the residuals' and coordinates' scales (ic, ix
+// their inverses).  The truncating sums come out 5e-8 (d >= 16) to 8e-8 (d = 2 to 5) small, measured
 // against 64 bits; the share kShare, under an ulp, moves three quarters of the
 // sums up by one and so gives the mean back.
 __device__ __forceinline__ void flush_g16(uint32_t tmem, uint32_t gcol, int B, int quarter, int half,
-                                          int lane, int d, int dp, int64_t n, float scale4, float gs, float ss,
+                                          int lane, int d, int dp, int64_t n, float scale4, float ic, const float *ix,
                                           float *__restrict__ grad, float *__restrict__ S) {
     constexpr float kShare = 5.0e-8f;
     const uint32_t tl = tmem + ((uint32_t)(32 * quarter) << 16) + gcol;
     const float s = tmem_ld1(tl + (uint32_t)dp);
     const int64_t row = (int64_t)B * TM + 32 * quarter + lane;
     const int hw = dp >> 1;
-    const float f = -scale4 * gs, fs = f * kShare;
+    const float f = -scale4 * ic;
     for (int c = 0; c < hw; c += 16) {
         float v[16];
         tmem_ld16(tl + (uint32_t)(half * hw + c), v);
         const int c0 = half * hw + c;
         if (row < n) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) v[q] = fmaf(v[q], f, v[q] * fs);
+            for (int q = 0; q < 16; q += 2) {
+                const float2 u = __fmul2_rn(make_float2(v[q], v[q + 1]), *reinterpret_cast<const float2 *>(ix + c0 + q));
+                const float2 o = __ffma2_rn(u, make_float2(f, f), __fmul2_rn(u, make_float2(f * kShare, f * kShare)));
+                v[q] = o.x;
+                v[q + 1] = o.y;
+            }
             float *gr = grad + row * d + c0;
             if ((d & 3) == 0 && c0 + 16 <= d) {
 #pragma unroll
@@ -508,7 +630,7 @@ __device__ __forceinline__ void flush_g16(uint32_t tmem, uint32_t gcol, int B, i
             }
         }
     }
-    if (half == 0 && row < n) atomicAdd(S + row, fmaf(s, ss, s * (ss * kShare)));
+    if (half == 0 && row < n) atomicAdd(S + row, fmaf(s, ic, s * (ic * kShare)));
 }
 
 // The same from the centre, one element at a time (any d, any alignment of x).
@@ -549,6 +671,18 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
+// The residuals of four columns from the accumulators' sums v (FP16):
+// r_ij = a_i + a_j - odd w_i w_j v with wi = -odd w_i, two columns per packed
+// operation.
+__device__ __forceinline__ void residuals4(float *v, float4 aj, float4 wj, float ai, float wi) {
+    const float2 a2 = make_float2(ai, ai), w2 = make_float2(wi, wi);
+    const float2 r0 = __ffma2_rn(__fmul2_rn(make_float2(v[0], v[1]), w2), make_float2(wj.x, wj.y),
+                                 __fadd2_rn(a2, make_float2(aj.x, aj.y)));
+    const float2 r1 = __ffma2_rn(__fmul2_rn(make_float2(v[2], v[3]), w2), make_float2(wj.z, wj.w),
+                                 __fadd2_rn(a2, make_float2(aj.z, aj.w)));
+    v[0] = r0.x; v[1] = r0.y; v[2] = r1.x; v[3] = r1.y;
+}
+
 // The backward kernel (gradient): 128 x 128 tiles, GEMM1 then GEMM2.  With
 // `partials` it also sums the loss from the same residual tiles (one FP64
 // partial per CTA): loss and gradient in one pass.
@@ -560,8 +694,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                       float *__restrict__ S, const float *__restrict__ a, int64_t n, int d, int nb,
                       int gx, int64_t T, int64_t nchunks, const int64_t *__restrict__ start,
                       float scale4, float *__restrict__ grad, double *__restrict__ partials, int qshift, int dg,
-                      const uint32_t *__restrict__ mx) {
-    // d: coordinates in the operands (a multiple of 32), dg: in grad.
+                      const float *__restrict__ w, const Stats *__restrict__ st) {
+    // d: coordinates in the operands (a multiple of 32), dg: in grad; w, st: FP16.
     // GEMM1 accumulators: two, used in turn (BF16), or one pair hi.hi | rest (F16)
     constexpr uint32_t kAcc = F16 ? 1 : 2;
     using Walk = ChunkWalk<MAP>;
@@ -602,6 +736,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         prefetch_map(&mTh);
         prefetch_map(&mTl);
     }
+    if (F16 && tid < kMaxDim) ctl.ix[tid] = __ldg(st->ix + tid);
     if (warp == 1) tmem_alloc(smem_u32(&ctl.tmem), kTmemCols);
     tc_fence_before();
     __syncthreads();
@@ -779,30 +914,36 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int quarter = warp & 3;            // TMEM lanes 32*quarter .. +31
         const int half = ew >> 2;                // columns [64*half, 64*half + 64)
         const int r = 32 * quarter + lane;       // this thread's row in the tile
-        float *ac = &ctl.acol[ew][0];
+        float *ac = &ctl.acol[ew][0], *wc = &ctl.wcol[ew][0];
         const int ngx = gx_buffers(NG);
         unsigned char *rowh = cbuf + half * TILE_BYTES + (r >> 3) * 1024 + (r & 7) * 128;
         unsigned char *rowl = rowh + 2 * TILE_BYTES;
-        Scales sc = {};
-        if (F16) sc = scales_of(mx, dg);
-        const float gs = sc.ix * sc.ic, ss = sc.ic;
+        // (FP16: the residuals come out in the scale of C)
+        const float ic = F16 ? __ldg(&st->ic) : 1.0f, odd = F16 ? -__ldg(&st->odd) * __ldg(&st->cs) : 0.0f;
         Walk walk(gx, nb, T, nchunks, start);
         uint32_t t = 0;
         int X, Y, pX = 0, pY = 0;
         bool have = walk.next(X, Y);
-        // a of the current tile's columns (va, vb) and row (vi), loaded a tile ahead
-        float va = 0.f, vb = 0.f, vi = 0.f;
+        // a of the current tile's columns (va, vb) and row (vi), loaded a tile
+        // ahead; FP16: and w, both once the C tile has left the registers
+        float va = 0.f, vb = 0.f, vi = 0.f, wa = 0.f, wb = 0.f, wr = 0.f;
         if (have) load_a(a, n, X, Y, half, r, lane, va, vb, vi);
+        if (F16 && have) load_a(w, n, X, Y, half, r, lane, wa, wb, wr);
         while (have && !*fail) {
             int Xn, Yn;
             const bool hn = walk.next(Xn, Yn);
             float na = 0.f, nbv = 0.f, ni = 0.f;
-            if (hn) load_a(a, n, Xn, Yn, half, r, lane, na, nbv, ni);
+            if (!F16 && hn) load_a(a, n, Xn, Yn, half, r, lane, na, nbv, ni);
             const uint32_t acc = t % kAcc, aph = (t / kAcc) & 1;
             const int64_t row0 = (int64_t)Y * TM, jb = (int64_t)X * TN + 64 * half;
-            __syncwarp();   // the previous tile's reads of ac are done
+            __syncwarp();   // the previous tile's reads of ac and wc are done
             ac[lane] = va;
             ac[lane + 32] = vb;
+            if (F16) {
+                wc[lane] = wa;
+                wc[lane + 32] = wb;
+            }
+            const float wi = wr * odd;
             const int64_t i = row0 + r;
             const float ai = vi;
             // valid columns q < lim: j < n, and j < i on a diagonal tile
@@ -819,10 +960,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (F16) {   // hi.hi, then the other products' accumulator
 #pragma unroll
                     for (int p = 0; p < 64; p += 32) {
-                        tmem_ld32(taddr + p, v0);
-                        tmem_ld32(taddr + TN + p, v1);
+                        tmem_ld64(taddr + p, v0, v1, TN);
 #pragma unroll
-                        for (int q = 0; q < 32; ++q) v[p + q] = ((v0[q] + v1[q]) * sc.is) * sc.id;
+                        for (int q = 0; q < 32; q += 2) {
+                            const float2 m = __fadd2_rn(make_float2(v0[q], v0[q + 1]), make_float2(v1[q], v1[q + 1]));
+                            v[p + q] = m.x;
+                            v[p + q + 1] = m.y;
+                        }
                     }
                 } else {
                     tmem_ld64(taddr, v0, v1);
@@ -837,11 +981,19 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int q = 0; q < 64; q += 4) {
                 const float4 aj = *reinterpret_cast<const float4 *>(ac + q);
                 const float al4[4] = {aj.x, aj.y, aj.z, aj.w};
+                if (F16) {
+                    residuals4(&v[q], aj, *reinterpret_cast<const float4 *>(wc + q), ai, wi);
+                    continue;
+                }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const float rq = (ai + al4[k]) - v[q + k];
                     v[q + k] = q + k < lim ? rq : 0.0f;
                 }
+            }
+            if (F16 && !__all_sync(0xffffffffu, lim == 64)) {
+#pragma unroll
+                for (int q = 0; q < 64; ++q) v[q] = q < lim ? v[q] : 0.0f;
             }
             if (partials) {   // the loss from the same residuals (loss and gradient in one pass)
                 float sq = 0.f;
@@ -857,8 +1009,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 uint32_t ph[4], pl[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const float f0 = F16 ? v[8 * c + 2 * k] * sc.c : v[8 * c + 2 * k],
-                                f1 = F16 ? v[8 * c + 2 * k + 1] * sc.c : v[8 * c + 2 * k + 1];
+                    const float f0 = v[8 * c + 2 * k], f1 = v[8 * c + 2 * k + 1];
                     if (F16) {
                         const __half2 hf = __floats2half2_rn(f0, f1);
                         const float2 b = __half22float2(hf);
@@ -878,16 +1029,20 @@ __global__ void __launch_bounds__(kThreads, 1)
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&ctl.cready));
+            if (F16 && hn) {
+                load_a(a, n, Xn, Yn, half, r, lane, na, nbv, ni);
+                load_a(w, n, Xn, Yn, half, r, lane, wa, wb, wr);
+            }
             if (t >= 1) {
                 // the previous tile's sides: its columns always, its rows at the end of a run
                 const uint32_t pb = (t - 1) % (uint32_t)ngx;
-                if (F16) flush_g16(tmem, kGY + NG * (1 + pb), pX, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+                if (F16) flush_g16(tmem, kGY + NG * (1 + pb), pX, quarter, half, lane, dg, d, n, scale4, ic, ctl.ix, grad, S);
                 else flush_g(tmem, kGY + NG * (1 + pb), pX, quarter, half, lane, d, n, scale4, grad, S);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctl.gxfree[pb]));
                 if (F16 || Y != pY) {
-                    if (F16) flush_g16(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+                    if (F16) flush_g16(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, ic, ctl.ix, grad, S);
                     else flush_g(tmem, kGY, pY, quarter, half, lane, d, n, scale4, grad, S);
                     tc_fence_before();
                     __syncwarp();
@@ -905,8 +1060,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
             const uint32_t gx0 = kGY + NG * (1 + (t - 1) % (uint32_t)ngx);
             if (F16) {
-                flush_g16(tmem, gx0, pX, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
-                flush_g16(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, gs, ss, grad, S);
+                flush_g16(tmem, gx0, pX, quarter, half, lane, dg, d, n, scale4, ic, ctl.ix, grad, S);
+                flush_g16(tmem, kGY, pY, quarter, half, lane, dg, d, n, scale4, ic, ctl.ix, grad, S);
             } else {
                 flush_g(tmem, gx0, pX, quarter, half, lane, d, n, scale4, grad, S);
                 flush_g(tmem, kGY, pY, quarter, half, lane, d, n, scale4, grad, S);
@@ -922,7 +1077,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (partials) {
         const double s = block_sum_ff<kThreads>(lhi, llo, ctl.red);
-        if (tid == 0) partials[blockIdx.x] = s;
+        const double ic = F16 ? (double)__ldg(&st->ic) : 1.0;
+        if (tid == 0) partials[blockIdx.x] = F16 ? s * ic * ic : s;
     }
 }
 
@@ -952,10 +1108,11 @@ struct Ctl2 {
     uint32_t tmem;
     int fail;
     alignas(16) float acol[kEpiWarps][TN];   // a_j of each epilogue warp's 128 columns
+    alignas(16) float wcol[kEpiWarps][TN];   // FP16: their w_j
     float red[2 * (kThreads / 32)];
 };
 
-constexpr int kCtl2Bytes = 8192;
+constexpr int kCtl2Bytes = 9216;
 constexpr int SMEM2 = 1024 + NS * STAGE + kCtl2Bytes;
 static_assert(sizeof(Ctl2) <= kCtl2Bytes, "control block");
 static_assert(SMEM2 <= 227 * 1024, "shared memory per block");
@@ -966,8 +1123,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     k_stress_umma_fwd(const __grid_constant__ CUtensorMap mPh, const __grid_constant__ CUtensorMap mPl,
                     const __grid_constant__ CUtensorMap mQh, const __grid_constant__ CUtensorMap mQl,
                     const float *__restrict__ a, int64_t n, int d, int nb, int nb2, int gx,
-                    int64_t total, double *__restrict__ partials, int qshift, int dg,
-                    const uint32_t *__restrict__ mx) {
+                    int64_t total, double *__restrict__ partials, int qshift, const float *__restrict__ w,
+                    const Stats *__restrict__ st) {
     // accumulators: two, used in turn (BF16), or one pair hi.hi | rest (F16)
     constexpr uint32_t kAcc = F16 ? 1 : 2;
     extern __shared__ unsigned char smem_raw[];
@@ -1083,9 +1240,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int quarter = warp & 3;            // TMEM lanes 32*quarter .. +31
         const int h = ew >> 2;                   // column block 2 sX + h: accumulator columns 128 h ..
         const int r = 32 * quarter + lane;       // this thread's row in the tile
-        float *ac = &ctl.acol[ew][0];
-        Scales sc = {};
-        if (F16) sc = scales_of(mx, dg);
+        float *ac = &ctl.acol[ew][0], *wc = &ctl.wcol[ew][0];
+        const float odd = F16 ? -__ldg(&st->odd) : 0.0f;
         SuperWalk<MAP> walk(gx, total, nb2);
         uint32_t t = 0;
         int sX, sY;
@@ -1098,8 +1254,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int q = 0; q < TN; q += 32) {
                 const int64_t j = jb + q + lane;
                 ac[q + lane] = j < n ? __ldg(a + j) : 0.0f;
+                if (F16) wc[q + lane] = j < n ? __ldg(w + j) : 0.0f;
             }
             const float ai = i < n ? __ldg(a + i) : 0.0f;
+            const float wi = F16 && i < n ? odd * __ldg(w + i) : 0.0f;   // M = odd w_i w_j times the sums
             // valid columns q < lim: j < n, j < i on a diagonal tile; none above
             // the diagonal or past the last block
             int64_t lim64 = (i < n && X <= Y && Y < nb) ? n - jb : 0;
@@ -1109,41 +1267,64 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!mbar_wait(smem_u32(&ctl.tfull[acc]), aph, fail, &g_error)) break;
             tc_fence_after();
             float sq = 0.f;
+            if (F16) {
+                // hi.hi and the other products' accumulator; both are free for the
+                // next step once their sums are in registers (the residuals' two
+                // factors per pair cost 7 of 110 us at n = 16384, d = 33 while the
+                // accumulators waited for them; 98 so)
+                const uint32_t taddr = tmem + acc * TN2 + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(TN * h);
+                float v[TN];
 #pragma unroll
-            for (int part = 0; part < 2; ++part) {
-                float v0[32], v1[32];
-                const uint32_t taddr = tmem + acc * TN2 + ((uint32_t)(32 * quarter) << 16) +
-                                       (uint32_t)(TN * h + 64 * part);
-                tmem_ld64(taddr, v0, v1);
-                if (F16) {   // the other products' accumulator, 32 columns at a time
-                    float w[32];
-                    tmem_ld32(taddr + TN2, w);
+                for (int c0 = 0; c0 < TN; c0 += 16) {
+                    float v0[16], v1[16];
+                    tmem_ld16(taddr + c0, v0);
+                    tmem_ld16(taddr + TN2 + c0, v1);
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) v0[q] = ((v0[q] + w[q]) * sc.is) * sc.id;
-                    tmem_ld32(taddr + TN2 + 32, w);
-#pragma unroll
-                    for (int q = 0; q < 32; ++q) v1[q] = ((v1[q] + w[q]) * sc.is) * sc.id;
+                    for (int q = 0; q < 16; ++q) v[c0 + q] = v0[q] + v1[q];
                 }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[acc]));
+                float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int q = 0; q < 32; q += 4) {
-                    const int c0 = 64 * part + q;
-                    const float4 a0 = *reinterpret_cast<const float4 *>(ac + c0);
-                    const float4 a1 = *reinterpret_cast<const float4 *>(ac + c0 + 32);
-                    const float x0[4] = {a0.x, a0.y, a0.z, a0.w}, x1[4] = {a1.x, a1.y, a1.z, a1.w};
+                for (int q = 0; q < TN; q += 4) {
+                    residuals4(&v[q], *reinterpret_cast<const float4 *>(ac + q), *reinterpret_cast<const float4 *>(wc + q),
+                               ai, wi);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        float r0 = (ai + x0[k]) - v0[q + k];
-                        float r1 = (ai + x1[k]) - v1[q + k];
-                        r0 = c0 + k < lim ? r0 : 0.0f;
-                        r1 = c0 + 32 + k < lim ? r1 : 0.0f;
-                        sq = fmaf(r0, r0, sq);
-                        sq = fmaf(r1, r1, sq);
+                    for (int k = 0; k < 4; k += 2) {
+                        const float2 r2 = make_float2(q + k < lim ? v[q + k] : 0.0f, q + k + 1 < lim ? v[q + k + 1] : 0.0f);
+                        s2 = __ffma2_rn(r2, r2, s2);
                     }
                 }
+                sq = s2.x + s2.y;
+            } else {
+#pragma unroll
+                for (int part = 0; part < 2; ++part) {
+                    float v0[32], v1[32];
+                    const uint32_t taddr = tmem + acc * TN2 + ((uint32_t)(32 * quarter) << 16) +
+                                           (uint32_t)(TN * h + 64 * part);
+                    tmem_ld64(taddr, v0, v1);
+#pragma unroll
+                    for (int q = 0; q < 32; q += 4) {
+                        const int c0 = 64 * part + q;
+                        const float4 a0 = *reinterpret_cast<const float4 *>(ac + c0);
+                        const float4 a1 = *reinterpret_cast<const float4 *>(ac + c0 + 32);
+                        const float x0[4] = {a0.x, a0.y, a0.z, a0.w}, x1[4] = {a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            float r0 = (ai + x0[k]) - v0[q + k];
+                            float r1 = (ai + x1[k]) - v1[q + k];
+                            r0 = c0 + k < lim ? r0 : 0.0f;
+                            r1 = c0 + 32 + k < lim ? r1 : 0.0f;
+                            sq = fmaf(r0, r0, sq);
+                            sq = fmaf(r1, r1, sq);
+                        }
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[acc]));
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[acc]));
             add_ff(lhi, llo, sq, 0.f);
             ++t;
         }
@@ -1164,88 +1345,130 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace f256
 
-// hi and lo of a value, BF16 or (F16) FP16 of a scaled value.
-template <bool F16>
+// hi and lo of a value, BF16 and FP16 (of a scaled value).
 __device__ __forceinline__ void split_float(float v, uint16_t &h, uint16_t &l) {
-    if (F16) {
-        const __half hh = __float2half_rn(v);
-        h = __half_as_ushort(hh);
-        l = __half_as_ushort(__float2half_rn(v - __half2float(hh)));
-    } else {
-        const __nv_bfloat16 hh = __float2bfloat16_rn(v);
-        h = __bfloat16_as_ushort(hh);
-        l = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(hh)));
-    }
+    const __nv_bfloat16 hh = __float2bfloat16_rn(v);
+    h = __bfloat16_as_ushort(hh);
+    l = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(hh)));
+}
+
+__device__ __forceinline__ void split_half(float v, uint16_t &h, uint16_t &l) {
+    const __half hh = __float2half_rn(v);
+    h = __half_as_ushort(hh);
+    l = __half_as_ushort(__float2half_rn(v - __half2float(hh)));
 }
 
 // P = [S | Delta], Q = [Delta | S] (hi, lo; rows of 2 dp; Q only when Qh is
-// given), a = S . Delta in FP32, and for the backward pass X^T hi, lo (rows
+// given), a = S . Delta in FP32 (FP16 backward: in the scale of C), and for the backward pass X^T hi, lo (rows
 // t < d: coordinates; row dp: ones; the others up to NG - 1: zeros; row pitch
 // `pitch`).  dp = d for BF16; for FP16 (F16) the next multiple of 32, the
-// columns beyond d zero.  32 points per block.
+// columns beyond d zero, and the points' w; block 0 leaves the main kernel's
+// scales in st.  32 points per block.
 template <bool F16>
 __global__ void __launch_bounds__(256) k_stress_prep(const float *__restrict__ x,
                                                      const float *__restrict__ y, int64_t n, int d, int dp,
-                                                     int NG, int64_t pitch, const uint32_t *__restrict__ mx,
-                                                     const float *__restrict__ c,
+                                                     int NG, int64_t pitch, Stats *st,
                                                      uint16_t *__restrict__ Ph,
                                                      uint16_t *__restrict__ Pl,
                                                      uint16_t *__restrict__ Qh,
                                                      uint16_t *__restrict__ Ql,
                                                      uint16_t *__restrict__ Th,
                                                      uint16_t *__restrict__ Tl,
-                                                     float *__restrict__ a, float *__restrict__ grad,
-                                                     float *__restrict__ S_) {
+                                                     float *__restrict__ a, float *__restrict__ w,
+                                                     float *__restrict__ grad, float *__restrict__ S_) {
     __shared__ float xs[32][97];
+    __shared__ Scales q;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i0 = (int64_t)blockIdx.x * 32;
-    Scales q = {};
-    if (F16) q = scales_of(mx, d);
     if (Th) {   // the backward adds into these
         const int64_t e0 = i0 * d, e1 = (i0 + 32 < n ? i0 + 32 : n) * d;
         for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) grad[e] = 0.f;
         if (threadIdx.x < 32 && i0 + threadIdx.x < n) S_[i0 + threadIdx.x] = 0.f;
     }
-    for (int p = warp; p < 32; p += 8) {
+    constexpr int K = kMaxDim / 32;
+    float xv[4][K], yv[4][K];   // FP16: the warp's points, loaded beside the scales
+    if (F16) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const int64_t i = i0 + warp + 8 * m;
+                const int t = lane + 32 * k;
+                const bool in = t < d && i < n;
+                xv[m][k] = in ? __ldg(x + i * d + t) : 0.f;
+                yv[m][k] = in ? __ldg(y + i * d + t) : 0.f;
+            }
+        if (warp == 0) find_scales(st, d, lane, q, blockIdx.x == 0 ? st : nullptr);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const int p = warp + 8 * m;
         const int64_t i = i0 + p;
         if (i >= n) break;
         float acc = 0.f;
-        for (int t = lane; t < dp; t += 32) {
-            const bool in = !F16 || t < d;
-            const float xv = in ? __ldg(x + i * d + t) : 0.f, yv = in ? __ldg(y + i * d + t) : 0.f;
-            const float ct = F16 && in ? __ldg(c + t) : 0.f;
-            const float S = F16 ? (xv - ct) + (yv - ct) : xv + yv, D = xv - yv;
-            uint16_t sh, sl, dh, dl;
-            if (F16) {
-                split_grid(S * q.s, sh, sl);
-                split_grid(D * q.d, dh, dl);
-            } else {
-                split_float<false>(S, sh, sl);
-                split_float<false>(D, dh, dl);
+        if (F16) {
+            float S[K], D[K], top = 0.f;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const int t = lane + 32 * k;
+                S[k] = D[k] = 0.f;
+                if (t >= d) continue;
+                const float ct = st->c[t], s = (xv[m][k] - ct) + (yv[m][k] - ct), e = xv[m][k] - yv[m][k];
+                acc = fmaf(s, e, acc);
+                xs[p][t] = xv[m][k] - ct;
+                S[k] = s * q.s[t];
+                D[k] = e * q.d[t];
+                top = fmaxf(top, fmaxf(fabsf(S[k]), fabsf(D[k])));
             }
-            const int64_t o = i * 2 * dp + t;
-            Ph[o] = sh; Pl[o] = sl; Ph[o + dp] = dh; Pl[o + dp] = dl;
-            if (Qh) { Qh[o] = dh; Ql[o] = dl; Qh[o + dp] = sh; Ql[o + dp] = sl; }
-            acc = fmaf(S, D, acc);
-            xs[p][t] = F16 ? xv - ct : xv;
+            top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top)));
+            const int e = max(exponent_of(top, 0), -100);
+            const float g = pow2(11 - e);
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const int t = lane + 32 * k;
+                if (t >= dp) continue;
+                uint16_t sh, sl, dh, dl;
+                split_grid(S[k] * g, sh, sl);
+                split_grid(D[k] * g, dh, dl);
+                const int64_t o = i * 2 * dp + t;
+                Ph[o] = sh; Pl[o] = sl; Ph[o + dp] = dh; Pl[o + dp] = dl;
+                if (Qh) { Qh[o] = dh; Ql[o] = dl; Qh[o + dp] = sh; Ql[o + dp] = sl; }
+                if (t >= d) xs[p][t] = 0.f;
+            }
+            if (lane == 0) w[i] = pow2(e - 11 + q.half);
+        } else {
+            for (int t = lane; t < d; t += 32) {
+                const float xv = __ldg(x + i * d + t), yv = __ldg(y + i * d + t);
+                const float S = xv + yv, D = xv - yv;
+                uint16_t sh, sl, dh, dl;
+                split_float(S, sh, sl);
+                split_float(D, dh, dl);
+                const int64_t o = i * 2 * dp + t;
+                Ph[o] = sh; Pl[o] = sl; Ph[o + dp] = dh; Pl[o + dp] = dl;
+                if (Qh) { Qh[o] = dh; Ql[o] = dl; Qh[o + dp] = sh; Ql[o + dp] = sl; }
+                acc = fmaf(S, D, acc);
+                xs[p][t] = xv;
+            }
         }
         acc = warp_sum_f32(acc);
-        if (lane == 0) a[i] = acc;
+        if (lane == 0) a[i] = F16 && Th ? acc * q.cs : acc;
     }
+    __syncthreads();
     if (Th) {
-        __syncthreads();
         for (int e = threadIdx.x; e < NG * 32; e += 256) {
             const int t = e >> 5, p = e & 31;
             const int64_t i = i0 + p;
             if (i >= n) continue;
-            const float v = t < dp ? (F16 ? xs[p][t] * q.x : xs[p][t]) : (t == dp ? 1.0f : 0.0f);
-            split_float<F16>(v, Th[t * pitch + i], Tl[t * pitch + i]);
+            const float v = t < dp ? (F16 ? xs[p][t] * q.x[t] : xs[p][t]) : (t == dp ? 1.0f : 0.0f);
+            if (F16) split_half(v, Th[t * pitch + i], Tl[t * pitch + i]);
+            else split_float(v, Th[t * pitch + i], Tl[t * pitch + i]);
         }
     }
 }
 
 struct Layout {
-    int64_t Ph, Pl, Qh, Ql, Th, Tl, a, part, edm, deal, sums, mx, total, pitch;
+    int64_t Ph, Pl, Qh, Ql, Th, Tl, a, part, edm, deal, sums, w, stats, total, pitch;
 };
 
 // The backward's chunks of the tile sequence: q per CTA, about kChunk
@@ -1283,8 +1506,9 @@ static Layout layout_of(int64_t n, int64_t d, bool bwd, bool f16) {
                      align_up(8 * chunks_of(nb * (nb + 1) / 2, kMaxCtas), 1024);
     }
     L.sums = L.deal + deal_bytes;   // backward: the per-point sums S of the flushes
-    L.mx = L.sums + (bwd ? align_up(4 * n, 1024) : 0);   // F16: the maxima and the centre
-    L.total = L.mx + (f16 ? 1024 : 0);
+    L.w = L.sums + (bwd ? align_up(4 * n, 1024) : 0);
+    L.stats = L.w + (f16 ? align_up(4 * n, 1024) : 0);
+    L.total = L.stats + (f16 ? kStatsBytes : 0);
     return L;
 }
 
@@ -1329,23 +1553,23 @@ template <bool F16>
 static cudaError_t launch_bwd(int map, unsigned ctas, cudaStream_t s, const CUtensorMap *m, float *S,
                               const float *a, int64_t n, int d, int nb, int gx, int64_t T, int64_t nchunks,
                               const int64_t *start, float scale4, float *grad, double *partials, int qshift, int dg,
-                              const uint32_t *mx) {
+                              const float *w, const Stats *st) {
     if (map == MAP_LAMBDA)
         k_stress_umma_bwd<MAP_LAMBDA, F16><<<ctas, kThreads, SMEM_BYTES, s>>>(
             m[0], m[1], m[2], m[3], m[4], m[5], S, a, n, d, nb, gx, T, nchunks, start, scale4, grad,
-            partials, qshift, dg, mx);
+            partials, qshift, dg, w, st);
     else if (map == MAP_BBOX)
         k_stress_umma_bwd<MAP_BBOX, F16><<<ctas, kThreads, SMEM_BYTES, s>>>(
             m[0], m[1], m[2], m[3], m[4], m[5], S, a, n, d, nb, gx, T, nchunks, start, scale4, grad,
-            partials, qshift, dg, mx);
+            partials, qshift, dg, w, st);
     else if (map == MAP_RB)
         k_stress_umma_bwd<MAP_RB, F16><<<ctas, kThreads, SMEM_BYTES, s>>>(
             m[0], m[1], m[2], m[3], m[4], m[5], S, a, n, d, nb, gx, T, nchunks, start, scale4, grad,
-            partials, qshift, dg, mx);
+            partials, qshift, dg, w, st);
     else
         k_stress_umma_bwd<MAP_LINEAR, F16><<<ctas, kThreads, SMEM_BYTES, s>>>(
             m[0], m[1], m[2], m[3], m[4], m[5], S, a, n, d, nb, gx, T, nchunks, start, scale4, grad,
-            partials, qshift, dg, mx);
+            partials, qshift, dg, w, st);
     return cudaGetLastError();
 }
 
@@ -1381,7 +1605,7 @@ static cudaError_t chunk_starts(int map, int64_t total, int gx, int nb, int64_t 
 template <bool F16>
 static cudaError_t launch_fwd(int map, unsigned ctas, cudaStream_t s, const CUtensorMap *m, const float *a,
                               int64_t n, int d, int nb, int nb2, int gx, int64_t total, double *partials,
-                              int qshift, int dg, const uint32_t *mx) {
+                              int qshift, const float *w, const Stats *st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(kThreads);
@@ -1396,15 +1620,15 @@ static cudaError_t launch_fwd(int map, unsigned ctas, cudaStream_t s, const CUte
     cfg.numAttrs = 1;
     if (map == MAP_LAMBDA)
         return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_LAMBDA, F16>, m[0], m[1], m[2], m[3], a, n, d, nb,
-                                  nb2, gx, total, partials, qshift, dg, mx);
+                                  nb2, gx, total, partials, qshift, w, st);
     if (map == MAP_BBOX)
         return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_BBOX, F16>, m[0], m[1], m[2], m[3], a, n, d, nb,
-                                  nb2, gx, total, partials, qshift, dg, mx);
+                                  nb2, gx, total, partials, qshift, w, st);
     if (map == MAP_RB)
         return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_RB, F16>, m[0], m[1], m[2], m[3], a, n, d, nb,
-                                  nb2, gx, total, partials, qshift, dg, mx);
+                                  nb2, gx, total, partials, qshift, w, st);
     return cudaLaunchKernelEx(&cfg, f256::k_stress_umma_fwd<MAP_LINEAR, F16>, m[0], m[1], m[2], m[3], a, n, d, nb,
-                              nb2, gx, total, partials, qshift, dg, mx);
+                              nb2, gx, total, partials, qshift, w, st);
 }
 
 // Two-CTA clusters of the forward kernel that fit on the device at once (one
@@ -1484,8 +1708,8 @@ static int run(bool bwd, int64_t n, int64_t d, int64_t dp, const float *x, const
     auto bf = [&](int64_t off) { return reinterpret_cast<uint16_t *>(w + off); };
     float *a = reinterpret_cast<float *>(w + L.a);
     double *partials = reinterpret_cast<double *>(w + L.part);
-    uint32_t *mx = F16 ? reinterpret_cast<uint32_t *>(w + L.mx) : nullptr;
-    float *c = F16 ? reinterpret_cast<float *>(w + L.mx + 16) : nullptr;
+    Stats *stats = F16 ? reinterpret_cast<Stats *>(w + L.stats) : nullptr;
+    float *pw = F16 ? reinterpret_cast<float *>(w + L.w) : nullptr;
     const int NG = (int)dp + 16;
     // Q = [Delta | S] is P = [S | Delta] with its two halves swapped: where dp
     // is a multiple of the K chunk, Q's chunk c is P's chunk at column
@@ -1518,17 +1742,17 @@ static int run(bool bwd, int64_t n, int64_t d, int64_t dp, const float *x, const
     if ((st = cuda_status(cudaGetDevice(&dev)))) return st;
     if ((st = cuda_status(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))) return st;
     if (F16) {
-        k_stress_centre<<<1, 8 * kMaxDim, 0, s>>>(x, n, (int)d, c, mx);
+        k_stress_centre<<<1, 8 * kMaxDim, 0, s>>>(x, y, n, (int)d, stats);
         note_launches(1);
         if ((st = launch_status())) return st;
         const int64_t mb = (n * d + 1023) / 1024;   // four elements a thread, at most four blocks an SM
-        k_stress_max<<<(unsigned)(mb < 4 * sms ? mb : 4 * sms), 256, 0, s>>>(x, y, n * d, (int)d, c, mx);
+        k_stress_max<<<(unsigned)(mb < 4 * sms ? mb : 4 * sms), 256, 0, s>>>(x, y, n * d, (int)d, stats);
         note_launches(1);
         if ((st = launch_status())) return st;
     }
     k_stress_prep<F16><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(
-        x, y, n, (int)d, (int)dp, NG, L.pitch, mx, c, bf(L.Ph), bf(L.Pl), qview ? nullptr : bf(L.Qh),
-        qview ? nullptr : bf(L.Ql), bwd ? bf(L.Th) : nullptr, bwd ? bf(L.Tl) : nullptr, a, grad,
+        x, y, n, (int)d, (int)dp, NG, L.pitch, stats, bf(L.Ph), bf(L.Pl), qview ? nullptr : bf(L.Qh),
+        qview ? nullptr : bf(L.Ql), bwd ? bf(L.Th) : nullptr, bwd ? bf(L.Tl) : nullptr, a, pw, grad,
         reinterpret_cast<float *>(w + L.sums));
     note_launches(1);
     if ((st = launch_status())) return st;
@@ -1548,7 +1772,7 @@ static int run(bool bwd, int64_t n, int64_t d, int64_t dp, const float *x, const
         float *S = reinterpret_cast<float *>(w + L.sums);
         prof_begin(s);
         le = launch_bwd<F16>(map, (unsigned)ctas, s, m, S, a, n, (int)dp, (int)nb, (int)g.gx, T, nchunks, start,
-                             (float)(4.0 * gscale), grad, loss ? partials : nullptr, qshift, (int)d, mx);
+                             (float)(4.0 * gscale), grad, loss ? partials : nullptr, qshift, (int)d, pw, stats);
     } else {
         // two-CTA clusters over the map's grid of 256 x 256 super-blocks
         const int64_t nb2 = (nb + 1) / 2;
@@ -1561,7 +1785,7 @@ static int run(bool bwd, int64_t n, int64_t d, int64_t dp, const float *x, const
         ctas = 2 * clusters;
         prof_begin(s);
         le = launch_fwd<F16>(map, (unsigned)ctas, s, m, a, n, (int)dp, (int)nb, (int)nb2, (int)g2.gx, total2,
-                             partials, qshift, (int)d, mx);
+                             partials, qshift, pw, stats);
     }
     prof_end(s);
     note_launches(1);
@@ -1570,7 +1794,7 @@ static int run(bool bwd, int64_t n, int64_t d, int64_t dp, const float *x, const
     if (!bwd) return reduce_partials(partials, ctas, partials + kMaxCtas, loss, s);
     const float *S = reinterpret_cast<const float *>(w + L.sums);
     if (F16) {
-        k_stress_sx_centred<<<(unsigned)((n * d + 255) / 256), 256, 0, s>>>(x, c, S, n, (int)d, (float)(4.0 * gscale), grad);
+        k_stress_sx_centred<<<(unsigned)((n * d + 255) / 256), 256, 0, s>>>(x, stats->c, S, n, (int)d, (float)(4.0 * gscale), grad);
     } else {
         const int64_t f4 = n * d / 4;
         k_stress_sx<<<(unsigned)((f4 + 255) / 256), 256, 0, s>>>(x, S, n, (int)d, (float)(4.0 * gscale), grad);

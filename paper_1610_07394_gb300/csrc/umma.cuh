@@ -396,7 +396,7 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
 }
 
 // 64 consecutive FP32 columns of this thread's TMEM lane: two loads, one wait.
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v0)[32], float (&v1)[32]) {
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v0)[32], float (&v1)[32], uint32_t second = 32) {
     uint32_t r[64];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -419,7 +419,7 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v0)[32], float
           "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
           "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]),
           "=r"(r[62]), "=r"(r[63])
-        : "r"(taddr + 32));
+        : "r"(taddr + second));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int t = 0; t < 32; ++t) {
