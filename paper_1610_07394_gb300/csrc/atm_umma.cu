@@ -354,10 +354,21 @@ __device__ __forceinline__ void add_square(float d, float &s, float &sl) {
     sl += e + ml;
 }
 
+// Points whose squared distance overflows FP32: both powers are 0, as 1 / s
+// is.  (s = infinity would leave NaN in the residuals below; NaN itself stays.)
+constexpr float kFar = 3.0e38f;
+
+__device__ __forceinline__ float inv_root(float &s, float &sl) {
+    const bool far = s > kFar;
+    s = far ? 1.0f : s;
+    sl = far ? 0.0f : sl;
+    return far ? 0.0f : rsqrtf(s);
+}
+
 // s^-1/2 and s^-3/2 of s + sl: the hardware estimate r and its residual
 // t = 1 - (s + sl) r^2 (formed without rounding s r).
 __device__ __forceinline__ void inv_powers(float s, float sl, float &r1, float &r3) {
-    const float r = rsqrtf(s);
+    const float r = inv_root(s, sl);
     const float u = s * r, ul = fmaf(s, r, -u);
     const float t = fmaf(-fmaf(sl, r, ul), r, fmaf(-u, r, 1.0f));
     r1 = fmaf(0.5f * t, r, r);
@@ -408,7 +419,7 @@ __device__ __forceinline__ UnitFF unit_ff(float xi, float yi, float zi, float xj
         two_sum(s, m, s, e);
         sl += e + ml;
     }
-    const float r = rsqrtf(s);
+    const float r = inv_root(s, sl);
     const float q = s * r, ql = fmaf(s, r, -q);
     const float t = fmaf(-fmaf(sl, r, ql), r, fmaf(-q, r, 1.0f));
     float r2, r2l;
