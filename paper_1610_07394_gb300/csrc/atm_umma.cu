@@ -354,21 +354,14 @@ __device__ __forceinline__ void add_square(float d, float &s, float &sl) {
     sl += e + ml;
 }
 
-// Points whose squared distance overflows FP32: both powers are 0, as 1 / s
-// is.  (s = infinity would leave NaN in the residuals below; NaN itself stays.)
+// Squares of distances that overflow FP32 (or nearly): R is 0 there, as 1 / s
+// is, but s = infinity would leave NaN in the residuals of s r^2.
 constexpr float kFar = 3.0e38f;
-
-__device__ __forceinline__ float inv_root(float &s, float &sl) {
-    const bool far = s > kFar;
-    s = far ? 1.0f : s;
-    sl = far ? 0.0f : sl;
-    return far ? 0.0f : rsqrtf(s);
-}
 
 // s^-1/2 and s^-3/2 of s + sl: the hardware estimate r and its residual
 // t = 1 - (s + sl) r^2 (formed without rounding s r).
 __device__ __forceinline__ void inv_powers(float s, float sl, float &r1, float &r3) {
-    const float r = inv_root(s, sl);
+    const float r = rsqrtf(s);
     const float u = s * r, ul = fmaf(s, r, -u);
     const float t = fmaf(-fmaf(sl, r, ul), r, fmaf(-u, r, 1.0f));
     r1 = fmaf(0.5f * t, r, r);
@@ -376,8 +369,9 @@ __device__ __forceinline__ void inv_powers(float s, float sl, float &r1, float &
     r3 = fmaf(1.5f * t, c, c);
 }
 
-// Unit vector (softened) u = p s^-1/2, s^-1/2 and s^-3/2 of p.
-__device__ __forceinline__ void unit_of(float x, float y, float z, float eps, float &ux, float &uy, float &uz, float &r1,
+// Unit vector (softened) u = p s^-1/2, s^-1/2 and s^-3/2 of p; false (and
+// nothing of use) beyond kFar.
+__device__ __forceinline__ bool unit_of(float x, float y, float z, float eps, float &ux, float &uy, float &uz, float &r1,
                                         float &r3) {
     float s = eps, sl = 0.f;
     add_square(z, s, sl);
@@ -387,6 +381,7 @@ __device__ __forceinline__ void unit_of(float x, float y, float z, float eps, fl
     ux = x * r1;
     uy = y * r1;
     uz = z * r1;
+    return !(s > kFar);
 }
 
 // (hi, lo) products and sums: the pair terms are formed to about twice FP32's
@@ -419,7 +414,10 @@ __device__ __forceinline__ UnitFF unit_ff(float xi, float yi, float zi, float xj
         two_sum(s, m, s, e);
         sl += e + ml;
     }
-    const float r = inv_root(s, sl);
+    const bool far = s > kFar;   // (a NaN is not)
+    s = far ? 1.0f : s;
+    sl = far ? 0.0f : sl;
+    const float r = far ? 0.0f : rsqrtf(s);
     const float q = s * r, ql = fmaf(s, r, -q);
     const float t = fmaf(-fmaf(sl, r, ql), r, fmaf(-q, r, 1.0f));
     float r2, r2l;
@@ -505,8 +503,9 @@ __global__ void __launch_bounds__(kNearThreads) k_atm_near(int64_t n, const floa
             if (nk == j || nj == k) ok = ok && key < pair_key(j, k);
             float bx, by, bz, cx, cy, cz;   // b = x_j - x_k, c = x_i - x_k
             float rb, Rb, rc, Rc;
-            unit_of(xj - K.x, yj - K.y, zj - K.z, eps, bx, by, bz, rb, Rb);
-            unit_of(xi - K.x, yi - K.y, zi - K.z, eps, cx, cy, cz, rc, Rc);
+            // (triples with a far point are 0)
+            ok &= unit_of(xj - K.x, yj - K.y, zj - K.z, eps, bx, by, bz, rb, Rb);
+            ok &= unit_of(xi - K.x, yi - K.y, zi - K.z, eps, cx, cy, cz, rc, Rc);
             const float al = fmaf(ax, bx, fmaf(ay, by, az * bz)), be = fmaf(bx, cx, fmaf(by, cy, bz * cz)),
                         ga = fmaf(ax, cx, fmaf(ay, cy, az * cz));
             const float R = ok ? Ra * Rb * Rc : 0.f;
@@ -734,7 +733,9 @@ __device__ __forceinline__ void columns16(const float (&v)[16], const float4 *co
         const bool ok = (valid >> e) & 1;
         const float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
         float s = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps)));
-        s = ok ? s : 1.0f;
+        // at kFar r3 is 0 and u finite, so all below is 0: overflowing squares,
+        // columns that are not pairs at any distance
+        s = ok ? fminf(s, kFar) : kFar;
         float r1, r3;
         inv_powers(s, 0.f, r1, r3);
         // (scales: powers of two, exact; columns that are not pairs may hold anything)
