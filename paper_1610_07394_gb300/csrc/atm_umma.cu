@@ -273,14 +273,11 @@ template <int MAP>
 __global__ void __launch_bounds__(256) k_atm_prep(int64_t n, const float *__restrict__ x, float eps, int ns,
                                                   int gx, int cells, bool rows, float *__restrict__ uinv,
                                                   int *__restrict__ nn,
-                                                  int *__restrict__ list, double *__restrict__ near_energy,
+                                                  int *__restrict__ list,
                                                   unsigned long long *__restrict__ pace, double *__restrict__ forces) {
     const int lane = threadIdx.x & 31;
     const int64_t gt = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (gt == 0) {
-        *near_energy = 0.0;
-        *pace = 0ull;
-    }
+    if (gt == 0) *pace = 0ull;
     if (gt < cells) {
         const int wy = (int)(gt / gx), wx = (int)(gt - (int64_t)wy * gx);
         const List2 L = decode2<MAP>((uint32_t)wx, (uint32_t)wy, ns);
@@ -464,7 +461,7 @@ template <bool FORCES>
 __global__ void __launch_bounds__(kNearThreads) k_atm_near(int64_t n, const float *__restrict__ x, float nu, float eps,
                                                            int seg, const float *__restrict__ uinv,
                                                            const int *__restrict__ nn,
-                                                           double *__restrict__ near_energy,
+                                                           double *__restrict__ partials,
                                                            double *__restrict__ forces) {
     __shared__ float4 xk[128];   // (x, y, z, nn) of up to 128 points
     __shared__ float red[2 * (kNearThreads / 32)];
@@ -556,9 +553,9 @@ __global__ void __launch_bounds__(kNearThreads) k_atm_near(int64_t n, const floa
         for (int c = 0; c < 6; ++c)
             atomicAdd(forces + 3 * (int64_t)(c < 3 ? i : j) + c % 3, (double)nu * ((double)fh[c] + (double)fl[c]));
     }
-    if (near_energy) {
+    if (partials) {
         const double s = block_sum_ff<kNearThreads>(eh, el, red);
-        if (tid == 0) atomicAdd(near_energy, (double)nu * s);
+        if (tid == 0) partials[blockIdx.x + (int64_t)gridDim.x * blockIdx.y] = (double)nu * s;
     }
 }
 
@@ -1093,8 +1090,15 @@ static cudaError_t launch(int clusters, cudaStream_t s, const CUtensorMap &mT, i
     return cudaLaunchKernelEx(&cfg, k_atm_umma<FORCES>, mT, n, x, nu, eps, W, list, uinv, nn, pace, partials, forces);
 }
 
+// Near pairs: 128 pairs by `seg` points per block, enough blocks for the chip.
+static int near_seg(int64_t n) { return n < 2048 ? 16 : n < 4096 ? 32 : 128; }
+static dim3 near_grid(int64_t n) {
+    return dim3((unsigned)((n + kNearThreads - 1) / kNearThreads), (unsigned)((n + near_seg(n) - 1) / near_seg(n)));
+}
+
 // Room behind the tables: the list of super-blocks, the row scales and the
-// FP64 partials (one per CTA and pass) with the reduction's slots.
+// FP64 partials (one per block of the near pairs, then one per CTA and pass,
+// summed in this order) with the reduction's slots.
 struct Rest {
     int64_t list, uinv, nn, pace, part, total;
 };
@@ -1107,8 +1111,9 @@ static Rest rest_of(int64_t n, int passes) {
     r.uinv = align_up(4 * (ns * (ns + 1) / 2), 256);
     r.nn = r.uinv + align_up(4 * n, 256);
     r.pace = r.nn + align_up(4 * n, 256);
-    r.part = r.pace + 16;   // [near pairs' energy][per CTA and pass]
-    r.total = r.part + 8 * (1 + (int64_t)kMaxCtas * passes + kReduceSlots);
+    r.part = r.pace + 16;
+    const dim3 g = near_grid(n);
+    r.total = r.part + 8 * ((int64_t)g.x * g.y + (int64_t)kMaxCtas * passes + kReduceSlots);
     return r;
 }
 
@@ -1169,7 +1174,9 @@ int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float ep
     int *list = (int *)(rb + R.list);
     float *uinv = (float *)(rb + R.uinv);
     int *nn = (int *)(rb + R.nn);
-    double *near_energy = (double *)(rb + R.part), *partials = near_energy + 1;
+    const dim3 ng = near_grid(n);
+    const int64_t nears = (int64_t)ng.x * ng.y;
+    double *near_part = (double *)(rb + R.part), *partials = near_part + nears;
     // operands (28 bytes per ordered pair) well beyond the 126 MB of L2 (n = 3000,
     // 252 MB: 1.56 ms without, 1.59 with; 4096: 3.77 both ways; 16384 above)
     unsigned long long *pace_ctr = (unsigned long long *)(rb + R.pace);
@@ -1181,14 +1188,12 @@ int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float ep
     const unsigned pb = (unsigned)((n + 7) / 8);
     double *fz = want_forces ? forces : nullptr;
     const bool rows = !want_forces && ns <= 24;
-    if (map == MAP_LAMBDA) k_atm_prep<MAP_LAMBDA><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, pace_ctr, fz);
-    else if (map == MAP_BBOX) k_atm_prep<MAP_BBOX><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, pace_ctr, fz);
-    else k_atm_prep<MAP_LINEAR><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, near_energy, pace_ctr, fz);
-    // near pairs: 128 pairs by `seg` points per block, enough blocks for the chip
-    const int seg = n < 2048 ? 16 : n < 4096 ? 32 : 128;
-    const dim3 ng((unsigned)((n + kNearThreads - 1) / kNearThreads), (unsigned)((n + seg - 1) / seg));
-    if (want_forces) k_atm_near<true><<<ng, kNearThreads, 0, s>>>(n, x, nu, eps, seg, uinv, nn, energy ? near_energy : nullptr, forces);
-    else k_atm_near<false><<<ng, kNearThreads, 0, s>>>(n, x, nu, eps, seg, uinv, nn, near_energy, nullptr);
+    if (map == MAP_LAMBDA) k_atm_prep<MAP_LAMBDA><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, pace_ctr, fz);
+    else if (map == MAP_BBOX) k_atm_prep<MAP_BBOX><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, pace_ctr, fz);
+    else k_atm_prep<MAP_LINEAR><<<pb, 256, 0, s>>>(n, x, eps, ns, (int)g2.gx, cells, rows, uinv, nn, list, pace_ctr, fz);
+    const int seg = near_seg(n);
+    if (want_forces) k_atm_near<true><<<ng, kNearThreads, 0, s>>>(n, x, nu, eps, seg, uinv, nn, energy ? near_part : nullptr, forces);
+    else k_atm_near<false><<<ng, kNearThreads, 0, s>>>(n, x, nu, eps, seg, uinv, nn, near_part, nullptr);
     note_launches(2);
     if ((st = launch_status())) return st;
     const int S = ns * (ns + 1) / 2;
@@ -1219,7 +1224,7 @@ int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float ep
         if ((st = launch_status())) return st;
     }
     if (!energy) return SIMPLEX_OK;
-    return reduce_partials(near_energy, 1 + (int64_t)2 * clusters * passes, partials + (int64_t)kMaxCtas * passes, energy, s);
+    return reduce_partials(near_part, nears + (int64_t)2 * clusters * passes, partials + (int64_t)kMaxCtas * passes, energy, s);
 }
 
 int atm_umma_errors(cudaStream_t s) {
