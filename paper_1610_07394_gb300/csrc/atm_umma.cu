@@ -677,8 +677,7 @@ __device__ __forceinline__ bool keep_pace(unsigned long long *ctr, unsigned long
 }
 
 struct Ctl {
-    uint64_t full[NS], empty[NS];   // ring: copies -> MMA -> copies
-    uint64_t pfull[NS];             // first CTA: the peer's copies of a stage have landed
+    uint64_t full[NS], empty[NS];   // ring: both CTAs' copies -> MMA (first CTA) -> copies (both)
     uint64_t tfull[kBufs], tempty[kBufs];   // accumulators: MMA -> both epilogues -> MMA (first CTA)
     uint64_t done;                  // every MMA of the block complete
     uint32_t tmem;
@@ -771,9 +770,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (tid == 0) {
         prefetch_map(&mT);
         for (int s = 0; s < NS; ++s) {
-            mbar_init(smem_u32(&ctl.full[s]), 1);
+            mbar_init(smem_u32(&ctl.full[s]), 2);
             mbar_init(smem_u32(&ctl.empty[s]), 1);
-            mbar_init(smem_u32(&ctl.pfull[s]), 1);
         }
         for (int b = 0; b < kBufs; ++b) {
             mbar_init(smem_u32(&ctl.tfull[b]), 1);
@@ -811,42 +809,47 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint32_t s = it % NS, ph = (it / NS) & 1;
                         // free once the pair's MMAs have read the stage
                         if (!(ok = mbar_wait(smem_u32(&ctl.empty[s]), ph ^ 1, fail, &g_error))) break;
-                        const uint32_t bar = smem_u32(&ctl.full[s]), dst = s_stages + s * STAGE;
+                        // the copies of both CTAs complete on the first one's barrier,
+                        // on which both arrive, also where one has none: neither gets
+                        // more than the ring ahead of the other
+                        const uint32_t bar = in_first(smem_u32(&ctl.full[s])), dst = s_stages + s * STAGE;
                         // an absent tile's rows or columns are not read out
                         const bool ha = has_tile(W.T, ra, c), hb = has_tile(W.T, rb, c);
-                        mbar_expect_tx(bar, (ha ? PAIR_BYTES : 0) + (hb ? PAIR_BYTES : 0));
+                        mbar_expect_tx_at(bar, (ha ? PAIR_BYTES : 0) + (hb ? PAIR_BYTES : 0));
                         if (ha)
-                            tma_load_2d(dst, &mT, 0, ((int)tile_slot(W.T, ra, c) * PLANES + pa) * 2 * TM, bar);
+                            tma2_load_2d(dst, &mT, 0, ((int)tile_slot(W.T, ra, c) * PLANES + pa) * 2 * TM, bar);
                         if (hb)
-                            tma_load_2d(dst + PAIR_BYTES, &mT, 0, ((int)tile_slot(W.T, rb, c) * PLANES + pb) * 2 * TM, bar);
+                            tma2_load_2d(dst + PAIR_BYTES, &mT, 0, ((int)tile_slot(W.T, rb, c) * PLANES + pb) * 2 * TM, bar);
                         ++it;
                     }
                 }
             }
-            // a failed block waits (bounded) for the loads it may have in flight
-            if (*fail)
-                for (uint32_t k = it > (uint32_t)NS ? it - NS : 0; k < it; ++k)
-                    mbar_drain(smem_u32(&ctl.full[k % NS]), (k / NS) & 1);
+            // a failed block waits (bounded) for the loads it may have in flight:
+            // the first CTA on its barriers, the second one, which cannot wait on
+            // those, a millisecond (a copy takes microseconds)
+            if (*fail) {
+                if (rank == 0) {
+                    for (uint32_t k = it > (uint32_t)NS ? it - NS : 0; k < it; ++k)
+                        mbar_drain(smem_u32(&ctl.full[k % NS]), (k / NS) & 1);
+                } else {
+                    const long long t0 = clock64();
+                    while (clock64() - t0 < 2000000) __nanosleep(1000);
+                }
+            }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer: the pair's first CTA issues for both (the
-        // whole warp, converged; one elected lane issues); the second one
-        // reports its landed stages
+        // whole warp, converged; one elected lane issues)
         const uint32_t id = idesc_f16(2 * TM, TN);
         Walk<UPPER> walk(W, list);
         uint32_t it = 0, u = 0;
         Seg g;
         bool ok = true;
-        while (ok && !*fail && walk.next(g)) {
+        while (rank == 0 && ok && !*fail && walk.next(g)) {
             const int stages = g.nt * (g.c1 - g.c0);
             for (int k = 0; k < stages; ++k, ++it) {
                 const uint32_t s = it % NS, ph = (it / NS) & 1;
                 if (!(ok = mbar_wait(smem_u32(&ctl.full[s]), ph, fail, &g_error))) break;
-                if (rank) {
-                    if (lane == 0) mbar_arrive_first(smem_u32(&ctl.pfull[s]));
-                    continue;
-                }
-                if (!(ok = mbar_wait(smem_u32(&ctl.pfull[s]), ph, fail, &g_error))) break;
                 const uint64_t d0 = sw128_desc(s_stages + s * STAGE);
                 // one accumulation of 64 k: the cross products first, while the
                 // sums are small, then hi.hi

@@ -311,10 +311,33 @@ __device__ __forceinline__ void tmem2_dealloc(uint32_t taddr, uint32_t cols) {
                  : "memory");
 }
 
-// Arrives on the mbarrier at `bar` of the cluster's first CTA.  What it hands
-// over is ordered by the tcgen05 fences (accumulators) or was complete before
-// (landed copies); a release at cluster scope would stall the warp for each
-// of its earlier memory accesses (a third of all stalls in the ATM kernel).
+// The address of `bar` in the cluster's first CTA.
+__device__ __forceinline__ uint32_t in_first(uint32_t bar) {
+    uint32_t ra;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(ra) : "r"(bar));
+    return ra;
+}
+
+// Arrival that expects `bytes` of copies, on a barrier of any CTA of the cluster.
+__device__ __forceinline__ void mbar_expect_tx_at(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
+// A copy into this CTA's shared memory that completes on a barrier of either
+// CTA of the pair (`bar`: see in_first).
+__device__ __forceinline__ void tma2_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+
+// Arrives on the mbarrier at `bar` of the cluster's first CTA, for accumulators
+// that have been read: tcgen05.wait::ld and the fence before it order those
+// reads ahead of the arrival, the waiter's tcgen05 fence its products behind it,
+// and nothing else is handed over.  A release at cluster scope would wait for
+// the warp's outstanding atomics (a third of all stalls in the ATM kernel).
 __device__ __forceinline__ void mbar_arrive_first(uint32_t bar) {
     asm volatile(
         "{\n\t.reg .b32 ra;\n\t"
