@@ -378,18 +378,32 @@ def atm_energy(x: torch.Tensor, nu=1.0, eps=1e-4, map="lambda") -> torch.Tensor:
     return ATMEnergy.apply(x, nu, eps, map)
 
 
+def _stress_workspace(op, n, d, map, prec):
+    """workspace(); where the device has no room for the tensor cores'
+    operands, what the FP32 kernels need (nothing for the gradient alone)."""
+    try:
+        return workspace(op, n, d, map, prec)
+    except torch.OutOfMemoryError:
+        rho = simplex_block_rho(op, d, prec)
+        if rho != simplex_block_rho(op, d, "fp32"):
+            raise   # BF16 has no other kernels
+        if op == "stress_bwd":
+            return None
+        return torch.empty(8 * (simplex_grid_blocks(2, -(-n // rho), map) + 1024), dtype=torch.uint8, device="cuda")
+
+
 def stress_fwd(x, y, map="lambda", prec="fp32", store_d=False):
     n, d = x.shape
     loss = torch.empty((), dtype=torch.float64, device=x.device)
     D = torch.empty(n * (n + 1) // 2, dtype=torch.float32, device=x.device) if store_d else None
-    simplex_stress_fwd(x, y, D, loss, map, prec, workspace("stress_fwd", n, d, map, prec))
+    simplex_stress_fwd(x, y, D, loss, map, prec, _stress_workspace("stress_fwd", n, d, map, prec))
     return loss, D
 
 
 def stress_bwd(x, y, gscale=1.0, map="lambda", prec="fp32"):
     n, d = x.shape
     grad = torch.empty_like(x)
-    simplex_stress_bwd(x, y, gscale, grad, map, prec, workspace("stress_bwd", n, d, map, prec))
+    simplex_stress_bwd(x, y, gscale, grad, map, prec, _stress_workspace("stress_bwd", n, d, map, prec))
     return grad
 
 
@@ -398,7 +412,7 @@ def stress_fwd_bwd(x, y, gscale=1.0, map="lambda", prec="fp32"):
     n, d = x.shape
     loss = torch.empty((), dtype=torch.float64, device=x.device)
     grad = torch.empty_like(x)
-    simplex_stress_fwd_bwd(x, y, gscale, grad, loss, map, prec, workspace("stress_fwd_bwd", n, d, map, prec))
+    simplex_stress_fwd_bwd(x, y, gscale, grad, loss, map, prec, _stress_workspace("stress_fwd_bwd", n, d, map, prec))
     return loss, grad
 
 

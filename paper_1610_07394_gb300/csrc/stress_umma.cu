@@ -1685,9 +1685,14 @@ static int64_t padded(int64_t d) { return (d + 31) / 32 * 32; }
 //             2560, 20: 44 and 66; 1500, 64: 40 and 50
 // n = 10000, d = 64: 79 against 575 us forward, 163 against 1125 us backward;
 // n = 20000, d = 96: 0.26 against 3.35 ms, 0.65 against 7.80 ms.
+// Up to 16 GB of operands and scan (n = 4 to 8 million): beyond, the scan's
+// 4 (n / 128)^2 bytes would refuse a call that the FP32 kernels take without.
+constexpr int64_t kF16MaxBytes = (int64_t)16 << 30;
+
 bool stress_f16_ok(int64_t n, int64_t d, bool bwd) {
     if (d > summa::kMaxDim || n < 1024) return false;
-    return (double)n * (double)n * (double)(d + 20) >= (bwd ? 1.5e8 : 3.6e8);
+    if ((double)n * (double)n * (double)(d + 20) < (bwd ? 1.5e8 : 3.6e8)) return false;
+    return stress_f16_workspace_bytes(n, d, bwd) <= kF16MaxBytes;
 }
 
 int64_t stress_f16_workspace_bytes(int64_t n, int64_t d, bool bwd) {
