@@ -68,6 +68,7 @@ FORCE_FLOPS_PER_TRIPLE = 53.5
 # products each: 150 flops for the energy (one side), 450 for the forces (three).
 CONTRACT_FLOPS_PER_TRIPLE = 150
 CONTRACT_FORCE_FLOPS_PER_TRIPLE = 450
+ATM_SUPER = 256   # points per side of the contraction's super-blocks of pairs
 FP32_LANES_PER_SM = 128
 L2_FLUSH_BYTES = 512 << 20
 PROFILES = os.path.join(ROOT, "profiles")
@@ -562,7 +563,7 @@ def row_atm_n3000(torch, sx, peaks):
     20, seed 7."""
     xh = synth.uniform_cube(3000, 3, 20.0, seed=7)
     r = _atm_row(torch, sx, peaks, torch.from_numpy(xh).cuda())
-    r["grid_blocks"] = {mp: sx.simplex_grid_blocks(3, -(-3000 // 32), mp) for mp in ("lambda", "bbox", "linear")}
+    r["super_block_grid"] = {mp: sx.simplex_grid_blocks(2, -(-3000 // ATM_SUPER), mp) for mp in ("lambda", "bbox", "linear")}
     r["cpu_baseline"] = _atm_cpu(xh, 4_000_000)
     return r
 
@@ -572,7 +573,7 @@ def row_atm_n12000(torch, sx, peaks):
     of side 20, seed 8: 2.88e11 triples."""
     xh = synth.uniform_cube(12000, 3, 20.0, seed=8)
     r = _atm_row(torch, sx, peaks, torch.from_numpy(xh).cuda(), steps=2)
-    r["grid_blocks"] = {mp: sx.simplex_grid_blocks(3, -(-12000 // 32), mp) for mp in ("lambda", "bbox", "linear")}
+    r["super_block_grid"] = {mp: sx.simplex_grid_blocks(2, -(-12000 // ATM_SUPER), mp) for mp in ("lambda", "bbox", "linear")}
     r["cpu_baseline"] = _atm_cpu(xh, 20_000_000)
     return r
 
@@ -645,6 +646,10 @@ def row_stress_n65536_d64(torch, sx, peaks):
     d = w["d"]
     r["fwd_tflops"] = 4 * d * r["fwd_lambda"] / 1e12
     r["bwd_tflops"] = 8 * d * r["bwd_lambda"] / 1e12
+    # issued as FP16 products: four of K = 2d, for the gradient three of N = d + 16
+    # per side as well, against the measured BF16 rate (the same pipe)
+    r["fwd_tensor_frac"] = 16 * d * r["fwd_lambda"] / 1e12 / peaks["bf16_tflops"]
+    r["bwd_tensor_frac"] = (16 * d + 12 * (d + 16)) * r["bwd_lambda"] / 1e12 / peaks["bf16_tflops"]
     r.update(_stress_tensor(torch, sx, peaks, x, y, ("lambda", "bbox", "linear", "rb")))
     w_ = host_cores()
     r["cpu_baseline"] = cpu_stress(xn, yn, list(range(n - 4 * w_, n)), w_)
@@ -947,8 +952,8 @@ def our_arm(args):
         torch.cuda.empty_cache()
     maps["lambda_vs_bbox"] = maps["lambda"] / maps["bbox"]
     maps["lambda_vs_linear"] = maps["lambda"] / maps["linear"]
-    maps["grid_blocks"] = {mp: sx.simplex_grid_blocks(3, -(-n // sx.simplex_block_rho("atm_forces")), mp)
-                           for mp in ("lambda", "bbox", "linear")}
+    maps["super_block_grid"] = {mp: sx.simplex_grid_blocks(2, -(-n // ATM_SUPER), mp)
+                                for mp in ("lambda", "bbox", "linear")}
     maps["steps_each"] = other
 
     # end to end through the public API with host buffers: the C ABI called

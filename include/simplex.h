@@ -98,8 +98,11 @@ const char *simplex_strerror(int status);
  * calling thread (0 if none). */
 int simplex_last_cuda_error(void);
 
-/* Block edge rho used by an operation (the library's tile size), for callers
- * that want nb = ceil(n / rho). */
+/* Block edge rho of an operation at its smallest sizes, for callers that want
+ * nb = ceil(n / rho); the workspaces' rules use it at every size.  Larger calls
+ * walk other blocks of the same maps: ATM as a contraction 256 (a 2-simplex of
+ * pairs), FP32 EDM 64 from n = 512 and 128 from n = 4608 (tiles 128 from 2560),
+ * FP32 stress on tensor cores 128 for the gradient and 256 for the loss. */
 int simplex_block_rho(int op, int64_t d, int prec);
 
 /*
@@ -245,7 +248,8 @@ int64_t simplex_edm_tiles_len(int64_t n);
  * pair matrices on the tensor cores, FP16 hi + lo splits of FP32 terms with
  * FP32 sums, over 256 x 256 super-blocks of pairs that the map's 2-simplex
  * grid lists, and the triples of each point's nearest neighbour one by one in
- * FP32; same accuracy or better, same workspace.
+ * FP32; same accuracy or better, same workspace.  The energy is a sum in a
+ * fixed order: the same bits from every call.
  */
 int simplex_atm_energy(int64_t n, int64_t d, const float *x, float nu, float eps,
                        double *energy, int map, void *workspace, int64_t ws_bytes,

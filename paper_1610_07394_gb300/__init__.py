@@ -116,7 +116,7 @@ def _prec(p) -> int:
 def _stream(stream=None) -> int:
     if stream is None:
         # torch.cuda.current_stream().cuda_stream without the Stream object
-        # (2 us of a small call's host time)
+        # (2.8 against 0.3 us of a small call's host time)
         return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 

@@ -159,7 +159,6 @@ __device__ __forceinline__ void planes_of(int o, int t, int &pa, int &pb) {
 struct Work {
     int S;        // super-blocks
     int G;        // products per segment of the outputs 6-8 (1, 2, 3 or 6)
-    int Kc;       // k chunks in all
     Table T;
 };
 
@@ -1145,8 +1144,8 @@ static int energy_passes(int64_t n, int64_t tab_bytes, int *cut) {
 
 // The contraction's fixed work (one 256 x 256 super-block per 256 points, six or
 // seven launches) pays from 640 points for the forces (n = 512: 88 against
-// 67 us, 640: 103 and 116, 1024: 152 and 297) and, as its tables take two or
-// three passes through the energy's smaller workspace, from 1280 for the energy
+// 67 us, 640: 103 and 116, 1024: 152 and 297) and, as its tables take two
+// passes through the energy's smaller workspace, from 1280 for the energy
 // (n = 1024: 131 against 106 us, 1152: 224 and 175, 1280: 191 and 214, 1536:
 // 224 and 326, 2048: 343 and 690).
 static constexpr int64_t kMinForces = 640, kMinEnergy = 1280;
@@ -1208,7 +1207,7 @@ int atm_umma_run(bool want_forces, int64_t n, const float *x, float nu, float ep
     const int64_t segs = (int64_t)S * (3 * (6 / G) + 7);
     if (clusters > segs) clusters = (int)segs;
     for (int p = 0; p < passes; ++p) {
-        const Work W = {S, G, Kc, Table{nrb, cut[p], cut[p + 1], want_forces ? 0 : 1}};
+        const Work W = {S, G, Table{nrb, cut[p], cut[p + 1], want_forces ? 0 : 1}};
         const dim3 tg((unsigned)(W.T.k1 - W.T.k0), (unsigned)nrb, TM / 32);
         unsigned char *tab = (unsigned char *)tables;
         if (want_forces) k_atm_tiles<false><<<tg, 256, 0, s>>>(n, x, eps, W.T, uinv, nn, tab);

@@ -1679,12 +1679,12 @@ static int64_t padded(int64_t d) { return (d + 31) / 32 * 32; }
 // Both paths measured: the launches around the main kernel (centre, maxima,
 // operands; the backward's tile scan) cost the F16 path 36 us forward and 40 us
 // backward at any size, the FP32 kernels grow with n^2 (d + 20):
-//   forward   n = 2561, d = 64: 40 against 53 us; 4096, 5: 34 and 42;
-//             2560, 20: 38 and 30; 3000, 3: 39 and 29
-//   backward  n = 2048, d = 64: 42 against 64 us; 3000, 3: 41 and 76;
-//             2560, 20: 44 and 66; 1500, 64: 40 and 50
-// n = 10000, d = 64: 79 against 575 us forward, 163 against 1125 us backward;
-// n = 20000, d = 96: 0.26 against 3.35 ms, 0.65 against 7.80 ms.
+//   forward   n = 2561, d = 64: 38 against 52 us; 4096, 5: 37 and 40; below the
+//             line 2560, 20: 38 and 29; 3000, 3: 39 and 27
+//   backward  n = 2048, d = 64: 39 against 64 us; 3000, 3: 42 and 75;
+//             2560, 20: 45 and 66; 1500, 64: 45 and 49
+// n = 10000, d = 64: 74 against 574 us forward, 161 against 1126 us backward;
+// n = 20000, d = 96: 0.22 against 3.35 ms, 0.67 against 7.80 ms.
 // Up to 16 GB of operands and scan (n = 4 to 8 million): beyond, the scan's
 // 4 (n / 128)^2 bytes would refuse a call that the FP32 kernels take without.
 constexpr int64_t kF16MaxBytes = (int64_t)16 << 30;
