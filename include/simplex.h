@@ -281,7 +281,8 @@ int simplex_atm_forces(int64_t n, int64_t d, const float *x, float nu, float eps
  * storing D.  loss: device, 1 double (written).
  * prec FP32: from about n^2 (d + 20) = 1.5e8 (gradient) or 3.6e8 (loss), d <= 96
  * and no d_out, the pair products run on the tensor cores from FP16 hi + lo
- * splits with FP32 sums, where the workspace has simplex_workspace_bytes(); with
+ * splits with FP32 sums, where the workspace has simplex_workspace_bytes() (up
+ * to 16 GB, n of 4 to 8 million; larger calls stay in FP32); with
  * less (8 bytes per grid block and 1024 for a loss, none for the gradient alone)
  * every step stays in FP32, the caller's choice.  The splits keep 22 bits of a
  * point's largest entry after every coordinate is scaled to one size: errors
